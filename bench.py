@@ -160,7 +160,7 @@ def interface_fraction(prof):
     return (prof["merge"] + prof["mortar"]) * 3 / prof["step"]
 
 
-def launches_per_step(mesh, viscous=0):
+def launches_per_step(mesh, viscous=0, stage_kernel=False):
     """Kernels of one captured SSP-RK3 step: on the side branch, beside the
     whole step, the merge of the next step's three stages (clocks and mortar
     tables), the launch forming their mortar offsets (Eq. xz) and the clock
@@ -168,9 +168,11 @@ def launches_per_step(mesh, viscous=0):
     the mortar flux when the mesh has an interface, in one launch) and the
     volume kernel (which sums the mortar contributions of its interface faces
     itself), plus for a viscous stage the common-solution face kernel (with
-    its mortar flux) and the gradient-trace kernel.  (Each sd_step call adds
-    the two launches merging its first step.)"""
-    per_stage = 2 + (2 if viscous else 0)
+    its mortar flux) and the gradient-trace kernel.  The FP32 forms on Euler
+    meshes run one launch per stage (stage_kernel).  (An sd_step call that
+    does not continue the steps before it adds the two launches merging its
+    first step.)"""
+    per_stage = 4 if viscous else (1 if stage_kernel else 2)
     return 3 + 3 * per_stage
 
 
@@ -816,7 +818,8 @@ def main():
             "cpu_baseline": cpu,
             "e2e": e2e,
             "clocks": clocks,
-            "gpu_launches": launches_per_step(w.mesh, w.params.viscous) * args.steps + 2,
+            "gpu_launches": launches_per_step(w.mesh, w.params.viscous,
+                                              prec in (ssd.SD_PREC_FP32, ssd.SD_PREC_FP32S)) * args.steps,
         }
         print(json.dumps(line))
     if world > 1:

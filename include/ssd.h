@@ -206,11 +206,13 @@ int sd_residual(sd_handle *h, double *R, int on_device);
 /* Advance nsteps steps of size dt with the SSP Runge-Kutta scheme chosen by
  * sd_params.rk_stages (Sec. 3: three stages at t, t + dt, t + dt/2; Sec. 4:
  * five stages); the mortar connectivity is rebuilt at every stage (Sec. 3.2).
- * Asynchronous: queued on the handle's stream as two kernel launches (the
- * stage clocks and mortar tables of the first step) and nsteps CUDA-graph
- * launches; each captured step also merges the next step's stages on a
- * second stream of the handle, beside its own kernels, and rejoins before it
- * ends, so the result is the same as merging each step after the last.
+ * Asynchronous: queued on the handle's stream as nsteps CUDA-graph launches,
+ * before them two kernel launches (the stage clocks and mortar tables of the
+ * first step) unless the call continues the steps before it with the same dt
+ * and an unchanged time; each captured step also merges the next step's
+ * stages on a second stream of the handle, beside its own kernels, and rejoins
+ * before it ends, so the result is the same as merging each step after the
+ * last.
  * Errors detected on the device are reported by sd_sync. */
 int sd_step(sd_handle *h, double dt, int nsteps);
 
@@ -295,7 +297,10 @@ int sd_batch_class_info(sd_batch *b, int i, int *info);
  * (the paper's "interface" work), ms[3] volume kernel (divergence, RK update,
  * traces); ms[4] = mean milliseconds per whole step.  The mortar flux is
  * timed as its own launch here; sd_step runs it inside the face launch of
- * the same pass.  Advances the solution by reps steps; synchronises. */
+ * the same pass.  On Euler meshes the FP32 forms take the conforming faces'
+ * fluxes inside the volume launch (ms[3]; there ms[1] is the boundary faces
+ * alone), and in sd_step the mortar and boundary fluxes too.  Advances the
+ * solution by reps steps; synchronises. */
 int sd_profile_step(sd_handle *h, double dt, int reps, double *ms);
 
 /* Measured FMA throughput of the current GPU in TFLOP/s (2 flops per FMA)

@@ -186,7 +186,22 @@ struct sd_handle {
   std::vector<int> zone_v, curved_v, iface_v;  // per element: zone, has an arc edge, has an interface face
   double *stage = nullptr;    // FP64 staging of host states (FP32 path)
   double *scratch = nullptr;  // device copy of a host residual
+  // the face-trace buffers; two where the stage kernel reads one and writes the
+  // other, else the same one twice
+  void *TRb[2] = {nullptr, nullptr};
+  // the trace buffer that holds (or will hold) the state's traces, and the
+  // stage-table set the next captured step reads; every stage, and so every
+  // step of 3 or 5 stages, moves on to the other one
+  int cur = 0;
   bool traces_valid = false;
+  // set cur holds the tables of a step of size tables_dt from the current time
+  // (the last captured step has merged them)
+  bool tables_valid = false;
+  double tables_dt = 0.0;
+  // per element face: 2 face + side, or the kind of a face that is not a
+  // conforming one (see ssd_stage.cuh)
+  std::vector<int> efmap;
+  bool in_batch = false;  // a batch's case: its kernels are the batch's (state and traces one variable at a time)
   // the captured step, one per set of stage tables it reads (see queue_step)
   cudaGraphExec_t step_exec[2] = {nullptr, nullptr};
   double graph_dt = 0.0;
@@ -489,6 +504,12 @@ int build_mesh(sd_handle *h, const sd_mesh *m, double omega1) {
   h->iface_v.assign(E, 0);
   for (int ef = 0; ef < 4 * E; ++ef)
     if (efi[ef] >= 0) h->iface_v[ef / 4] = 1;
+  h->efmap.assign(4 * (size_t)E, -1);
+  for (size_t k = 0; k < faces.size(); ++k) {
+    h->efmap[faces[k].x] = (int)(2 * k);
+    h->efmap[faces[k].y] = (int)(2 * k + 1);
+  }
+  for (const int4 &b : bfaces) h->efmap[b.x] = -2;
   cudaError_t ce;
   int4 *dfaces, *dbfaces, *dL, *dR;
   double *dcorn, *dLa, *dLw, *dLS, *dRa, *dRw, *dRS, *dLiW, *dRiW, *dcub = nullptr, *dzpar, *dLal, *dRal;
@@ -570,6 +591,27 @@ cudaError_t alloc_buffers(sd_handle *h, const std::vector<int> &zone, const std:
   if (otf && (e = dalloc(h, &md.egeo, w * Ep * 8))) return e;
   if (otf && (e = cudaMemsetAsync(md.egeo, 0, w * Ep * 8, h->stream))) return e;
   if ((e = dalloc(h, &md.TR, w * Ep * 16 * N))) return e;
+  h->TRb[0] = h->TRb[1] = md.TRo = md.TR;
+  md.frec = md.fgp = nullptr;
+  md.tord = nullptr;
+  if (const int epb = h->in_batch ? 0 : h->eng->stage_tile(md.viscous)) {
+    if ((e = dalloc(h, &h->TRb[1], w * Ep * 16 * N))) return e;
+    // tiles in working order: those with an interface or boundary face last
+    const int nt = (int)((E + epb - 1) / epb);
+    std::vector<char> late(nt, 0);
+    for (size_t ef = 0; ef < 4 * E; ++ef)
+      if (h->efmap[ef] < 0) late[ef / 4 / epb] = 1;
+    std::vector<int> order;
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int t = 0; t < nt; ++t)
+        if (late[t] == pass) order.push_back(t);
+      if (!pass) h->eng->set_early_tiles((int)order.size());
+    }
+    int *dord;
+    if ((e = upload(h, &dord, order.data(), order.size()))) return e;
+    md.tord = dord;
+    if ((e = cudaStreamSynchronize(h->stream))) return e;  // order leaves scope
+  }
   if ((e = dalloc(h, &md.CF, w * Ep * 16 * N))) return e;
   md.CQ = md.GTR = md.GSP = nullptr;
   if (md.viscous) {
@@ -634,6 +676,37 @@ cudaError_t alloc_buffers(sd_handle *h, const std::vector<int> &zone, const std:
   }
   // the host vectors above go out of scope: wait for their copies
   return cudaStreamSynchronize(h->stream);
+}
+
+// The stage kernel's face records (after the engine has formed the face
+// table).  A face needs its own per-point row where the normal or V_g.n varies
+// along it: on rotating zones and next to curved cells.
+cudaError_t build_face_records(sd_handle *h) {
+  MeshDev &md = h->md;
+  if (h->in_batch || !h->eng->stage_tile(md.viscous)) return cudaSuccess;
+  const size_t E = md.E, N = h->N, Ep = (E + kElemPad - 1) / kElemPad * kElemPad;
+  std::vector<char> varies(md.nF ? md.nF : 1, 0);
+  for (size_t ef = 0; ef < 4 * E; ++ef)
+    if (h->efmap[ef] >= 0 && (h->zone_v[ef / 4] || h->curved_v[ef / 4])) varies[h->efmap[ef] >> 1] = 1;
+  std::vector<int> row(4 * Ep, -1);
+  int rows = 0;
+  for (size_t ef = 0; ef < 4 * E; ++ef)
+    if (h->efmap[ef] >= 0 && varies[h->efmap[ef] >> 1]) row[ef] = rows++;
+  float4 *rec, *pts;
+  int *tmp = nullptr;
+  cudaError_t e;
+  if ((e = dalloc(h, &rec, sizeof(float4) * 4 * Ep))) return e;
+  if ((e = dalloc(h, &pts, sizeof(float4) * N * rows))) return e;
+  md.frec = rec;
+  md.fgp = pts;
+  if ((e = cudaMalloc(&tmp, sizeof(int) * 8 * Ep))) return e;
+  e = cudaMemcpyAsync(tmp, h->efmap.data(), sizeof(int) * 4 * E, cudaMemcpyHostToDevice, h->stream);
+  if (!e) e = cudaMemcpyAsync(tmp + 4 * Ep, row.data(), sizeof(int) * 4 * Ep, cudaMemcpyHostToDevice, h->stream);
+  if (!e) h->eng->face_records(md, tmp, tmp + 4 * Ep, (int)(4 * Ep), h->stream);
+  if (!e) e = cudaGetLastError();
+  if (!e) e = cudaStreamSynchronize(h->stream);
+  cudaFree(tmp);
+  return e;
 }
 
 // device flags: the OR of the primary clock's and the stage records' of both
@@ -737,6 +810,16 @@ MeshDev stage_view(const sd_handle *h, int k, int set = 0) {
   m.Lcount = sm.Lcount[k];
   m.Rstart = sm.Rstart[k];
   m.Rcount = sm.Rcount[k];
+  // a step that reads table set `set` also starts from trace buffer `set`
+  m.TR = h->TRb[(set + k) & 1];
+  m.TRo = h->TRb[(set + k + 1) & 1];
+  return m;
+}
+
+// the base view with the current traces (residuals)
+MeshDev base_view(const sd_handle *h) {
+  MeshDev m = h->md;
+  m.TR = m.TRo = h->TRb[h->cur];
   return m;
 }
 
@@ -815,13 +898,14 @@ int plan_step(sd_handle *h, double dt, BatchStageHost *plan, int ts) {
   return n;
 }
 
-// The clocks and tables of every stage of the step starting at t_n, into
-// set 0 (before the first captured step of a call; each captured step then
-// merges the next step into the other set).
+// The clocks and tables of every stage of the step starting at t_n, into the
+// set the next captured step reads (before the first captured step of a call
+// that does not continue the steps before it; each captured step then merges
+// the next step into the other set).
 void queue_merge_first(sd_handle *h, double dt) {
   BatchStageHost plan[kMaxStages];
-  const int n = plan_step(h, dt, plan, 0);
-  h->eng->merge_stages(h->md, h->sm, dt, 0, n, 0, 1024, h->stream);
+  const int n = plan_step(h, dt, plan, h->cur);
+  h->eng->merge_stages(h->md, h->cur ? h->sm_b : h->sm, dt, 0, n, 0, 1024, h->stream);
 }
 
 // One time step for capture, reading stage-table set ts.  The merges depend
@@ -852,7 +936,7 @@ extern "C" {
 
 const char *sd_create_error(void) { return g_create_error.c_str(); }
 
-int sd_create(const sd_mesh *m, int p, const sd_params *prm, sd_handle **out) {
+static int create_handle(const sd_mesh *m, int p, const sd_params *prm, bool in_batch, sd_handle **out) {
   g_create_error.clear();
   if (!out) return SD_ERR_ARG;
   *out = nullptr;
@@ -884,6 +968,7 @@ int sd_create(const sd_mesh *m, int p, const sd_params *prm, sd_handle **out) {
   h->E = m->n_elems;
   h->prm = *prm;
   h->precision = prm->precision;
+  h->in_batch = in_batch;
   cudaError_t ce;
   if (prm->stream) {
     h->stream = (cudaStream_t)prm->stream;
@@ -948,6 +1033,7 @@ int sd_create(const sd_mesh *m, int p, const sd_params *prm, sd_handle **out) {
   }
   if (!rc && (ce = h->eng->init(hb, h->md, h->stream))) rc = cuda_fail(h, ce, "engine init");
   if (!rc && (ce = cudaGetLastError())) rc = cuda_fail(h, ce, "geometry kernels");
+  if (!rc && (ce = build_face_records(h))) rc = cuda_fail(h, ce, "face records");
   if (!rc) {
     int flags = 0;
     rc = read_flags(h, &flags, false);
@@ -960,6 +1046,10 @@ int sd_create(const sd_mesh *m, int p, const sd_params *prm, sd_handle **out) {
   }
   *out = h;
   return SD_OK;
+}
+
+int sd_create(const sd_mesh *m, int p, const sd_params *prm, sd_handle **out) {
+  return create_handle(m, p, prm, false, out);
 }
 
 int sd_destroy(sd_handle *h) {
@@ -1043,6 +1133,7 @@ int sd_get_state(sd_handle *h, double *Q, int on_device) {
 int sd_set_time(sd_handle *h, double t) {
   if (!h || !std::isfinite(t)) return fail(h, SD_ERR_ARG, "bad time");
   cudaError_t e = cudaStreamSynchronize(h->stream);
+  h->tables_valid = false;
   if (!e) {
     h->h_pinned[0] = t;
     e = cudaMemcpyAsync(&h->md.clk->t_n, h->h_pinned, sizeof(double), cudaMemcpyHostToDevice, h->stream);
@@ -1071,9 +1162,10 @@ int sd_residual(sd_handle *h, double *R, int on_device) {
     dst = h->scratch;
   }
   const StatePtr none{nullptr, nullptr};
-  h->eng->trace(h->md, h->eng->A(), h->stream);
-  h->eng->couple(h->md, h->eng->A(), 0.0, 0.0, h->stream);
-  h->eng->volume(h->md, h->eng->A(), none, none, dst, RkArgs(), MODE_RESIDUAL, h->stream);
+  const MeshDev md = base_view(h);
+  h->eng->trace(md, h->eng->A(), h->stream);
+  h->eng->couple(md, h->eng->A(), 0.0, 0.0, h->stream);
+  h->eng->volume(md, h->eng->A(), none, none, dst, RkArgs(), MODE_RESIDUAL, h->stream);
   if ((e = cudaGetLastError())) return cuda_fail(h, e, "residual kernels");
   h->traces_valid = true;
   if (!on_device) {
@@ -1090,7 +1182,7 @@ int sd_step(sd_handle *h, double dt, int nsteps) {
   if (nsteps == 0) return SD_OK;
   cudaError_t e;
   if (!h->traces_valid) {
-    h->eng->trace(h->md, h->eng->A(), h->stream);
+    h->eng->trace(base_view(h), h->eng->A(), h->stream);
     if ((e = cudaGetLastError())) return cuda_fail(h, e, "trace kernel");
     h->traces_valid = true;
   }
@@ -1116,10 +1208,17 @@ int sd_step(sd_handle *h, double dt, int nsteps) {
     }
     h->graph_dt = dt;
   }
-  queue_merge_first(h, dt);
-  if ((e = cudaGetLastError())) return cuda_fail(h, e, "merge kernels");
-  for (int k = 0; k < nsteps; ++k)
-    if ((e = cudaGraphLaunch(h->step_exec[k & 1], h->stream))) return cuda_fail(h, e, "graph launch");
+  if (!(h->tables_valid && h->tables_dt == dt)) {
+    queue_merge_first(h, dt);
+    if ((e = cudaGetLastError())) return cuda_fail(h, e, "merge kernels");
+    h->tables_dt = dt;
+  }
+  h->tables_valid = false;
+  for (int k = 0; k < nsteps; ++k) {
+    if ((e = cudaGraphLaunch(h->step_exec[h->cur], h->stream))) return cuda_fail(h, e, "graph launch");
+    h->cur ^= 1;
+  }
+  h->tables_valid = true;  // merged beside the last step
   return SD_OK;
 }
 
@@ -1186,9 +1285,10 @@ int sd_profile_step(sd_handle *h, double dt, int reps, double *ms) {
   for (int k = 0; k < 6; ++k)
     if ((e = cudaEventCreate(&ev[k]))) return cuda_fail(h, e, "event");
   if (!h->traces_valid) {
-    h->eng->trace(h->md, h->eng->A(), h->stream);
+    h->eng->trace(base_view(h), h->eng->A(), h->stream);
     h->traces_valid = true;
   }
+  h->tables_valid = false;  // the time moves on without the captured steps' merges
   double acc[5] = {0, 0, 0, 0, 0};
   const double cs[3] = {0.0, 1.0, 0.5}, al[3] = {0.0, 0.75, 1.0 / 3.0}, be[3] = {1.0, 0.25, 2.0 / 3.0};
   // the mortar flux as its own launch, so that the interface work is timed
@@ -1202,18 +1302,21 @@ int sd_profile_step(sd_handle *h, double dt, int reps, double *ms) {
       const StatePtr qin = k == 0 ? A : B;
       const StatePtr qb = k == 0 ? none : A;
       const StatePtr qo = k == 2 ? A : B;
+      MeshDev m = base_view(h);
+      m.TRo = h->TRb[h->cur ^ 1];
       cudaEventRecord(ev[0], h->stream);
-      h->eng->clock_merge(h->md, cs[k], dt, h->stream);
+      h->eng->clock_merge(m, cs[k], dt, h->stream);
       cudaEventRecord(ev[1], h->stream);
-      h->eng->faces(h->md, qin, h->stream);
+      h->eng->faces(m, qin, h->stream);
       cudaEventRecord(ev[2], h->stream);
-      h->eng->mortars(h->md, h->stream);
+      h->eng->mortars(m, h->stream);
       cudaEventRecord(ev[3], h->stream);
       RkArgs rk;
       rk.has_base = k > 0;
       rk.a0 = al[k];
       rk.bdt = be[k] * dt;
-      h->eng->volume(h->md, qin, qb, qo, nullptr, rk, MODE_RK, h->stream);
+      h->eng->volume(m, qin, qb, qo, nullptr, rk, MODE_RK, h->stream);
+      h->cur ^= 1;
       cudaEventRecord(ev[4], h->stream);
       if ((e = cudaEventSynchronize(ev[4]))) break;
       for (int c = 0; c < 4; ++c) {
@@ -1323,7 +1426,10 @@ std::vector<std::vector<BatchStageHost>> class_stages(sd_batch *b, const sd_batc
     BatchStageHost plan[kMaxStages];
     double cc[kMaxStages];
     step_plan(h, dts[cl.members[c]], plan, cc);
-    for (int k = 0; k < b->nstages; ++k) st[k][c] = plan[k];
+    for (int k = 0; k < b->nstages; ++k) {
+      st[k][c] = plan[k];
+      st[k][c].md.TR = st[k][c].md.TRo = h->TRb[0];  // a face pass of its own reads the old traces first
+    }
   }
   return st;
 }
@@ -1482,7 +1588,7 @@ int sd_batch_create(int n, const sd_mesh *const *meshes, const int *p, const sd_
     sd_params pi = prm[i];
     pi.stream = nullptr;  // every case keeps its own stream for its own calls
     sd_handle *h = nullptr;
-    int rc = sd_create(meshes[i], p[i], &pi, &h);
+    int rc = create_handle(meshes[i], p[i], &pi, true, &h);
     if (rc) return fail_b(rc, "case " + std::to_string(i) + ": " + g_create_error);
     b->cases.push_back(h);
   }
@@ -1513,6 +1619,7 @@ int sd_batch_create(int n, const sd_mesh *const *meshes, const int *p, const sd_
       h->sm.n = b->nstages;
       for (int k = 0; k < b->nstages; ++k) {
         h->sm.c[k] = c[k];
+        plan[k].md.TR = plan[k].md.TRo = h->TRb[0];
         stage[(size_t)k * n + i] = plan[k].md;
       }
       base[i] = h->md;
@@ -1613,6 +1720,7 @@ int sd_batch_step(sd_batch *b, const double *dt, int nsteps) {
   }
   for (int i = 0; i < n; ++i) {
     sd_handle *h = b->cases[i];
+    h->tables_valid = false;  // the case's time moves on without its own captured steps
     if (!h->traces_valid) {
       h->eng->trace(h->md, h->eng->A(), b->stream);
       h->traces_valid = true;
@@ -1731,7 +1839,7 @@ int sd_residual_noalloc(sd_handle *h, double *R, int on_device) {
   cudaError_t e = noalloc_base(&base);
   if (e) return cuda_fail(h, e, "sd_residual_noalloc work memory address");
   unsigned char *b = (unsigned char *)base;
-  MeshDev md = md0;
+  MeshDev md = base_view(h);
   md.mLf = (int *)(b + o_mLf);
   md.mRf = (int *)(b + o_mRf);
   md.mgeo = (double *)(b + o_mgeo);

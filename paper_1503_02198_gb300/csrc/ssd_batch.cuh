@@ -47,7 +47,8 @@ __global__ void __launch_bounds__(FB) k_batch_faces(BatchWork w) {
   const int nmb = __ldg(w.nmb + c);
   if (!batch_check(md, lb >= 0 && nmb >= 0 && (lb < nmb || (lb - nmb) * FB < (md.nF + md.nB) * N))) return;
   if (lb < nmb) {
-    mortar_flux_body<T, N, MMODE, MortCfg<N>::MPB>(md, lb);
+    __shared__ MortShared<T, N, MMODE, MortCfg<N>::MPB> sh;
+    mortar_flux_body(md, lb, sh);
     return;
   }
   const int t = (lb - nmb) * FB + threadIdx.x;

@@ -540,6 +540,38 @@ struct ElemGeo {
       }
     }
   }
+  // the same for a cell of the stationary zone (z = 0), unrotated: load, and
+  // the metric vectors of a line (V_g is 0)
+  __device__ __forceinline__ void load_still(const MeshDev &md, int f, const T *r) {
+    int ti = ((f & ~kIfaceBit) >> kZoneBits) - 1;
+    if (!ssd_check(md, ti < md.nTab && (OTF || ti >= 0))) ti = 0;
+    tab = OTF && ti < 0 ? nullptr : (const T *)md.geo + (size_t)ti * L::G;
+    if (OTF) {
+      const float4 a = reinterpret_cast<const float4 *>(r)[0], b = reinterpret_cast<const float4 *>(r)[1];
+      e1x = a.z, e1y = a.w, e3x = b.x, e3y = b.y, dx = b.z, dy = b.w;
+    }
+  }
+  __device__ __forceinline__ void line_metrics_still(int d, int m, T *vx, T *vy) const {
+    if (OTF && tab == nullptr) {
+      // the tangent with the direction's sign, sg (A + u d): a sign commutes
+      // with every rounding
+      const T sg = d == 0 ? T(1) : T(-1);
+      const T Ax = sg * (d == 0 ? e3x : e1x), Ay = sg * (d == 0 ? e3y : e1y), Dx = sg * dx, Dy = sg * dy;
+#pragma unroll
+      for (int i = 1; i < N; ++i) {
+        const T u = cVB<T, N>.Xf[i];
+        vx[i] = Ay + u * Dy;
+        vy[i] = -(Ax + u * Dx);
+      }
+    } else {
+#pragma unroll
+      for (int i = 1; i < N; ++i) {
+        const int k = d == 0 ? L::ax + m * (N + 1) + i : L::bx + i * N + m;
+        vx[i] = tab[k];
+        vy[i] = tab[k + L::ay - L::ax];
+      }
+    }
+  }
   // metric vector of the end FP at point j of face f
   __device__ __forceinline__ void face(int f, int j, T &vx, T &vy, T &g) const {
     if (f == 1) xi_fp(N, j, vx, vy, g);
@@ -573,6 +605,17 @@ struct ElemGeo {
       return recip(mul_sub(xx, ye, xe, yx));
     }
     return ((const T *)md.geo + (size_t)ti * L::G)[L::iJ + j * N + i];
+  }
+  // the same at SP sp = j N + i with its coordinates (X_i, X_j) at hand: a warp's
+  // threads take different SPs, and constant memory serves one address at a time
+  static __device__ __forceinline__ T inv_jac_at(const MeshDev &md, int f, const T *r, int sp, T xi, T eta) {
+    const int ti = ((f & ~kIfaceBit) >> kZoneBits) - 1;
+    if (OTF && ti < 0) {
+      const float4 a = reinterpret_cast<const float4 *>(r)[0], b = reinterpret_cast<const float4 *>(r)[1];
+      const T xx = a.z + eta * b.z, yx = a.w + eta * b.w, xe = b.x + xi * b.z, ye = b.y + xi * b.w;
+      return recip(mul_sub(xx, ye, xe, yx));
+    }
+    return ((const T *)md.geo + (size_t)ti * L::G)[L::iJ + sp];
   }
   // gradients of xi and eta at SP (X_i, X_j): (xi_x, xi_y), (eta_x, eta_y)
   __device__ __forceinline__ void sp_grad(int i, int j, T &xix, T &xiy, T &etx, T &ety) const {
@@ -745,6 +788,8 @@ static __device__ void clock_merge_body(const MeshDev &md, int ii, double c, dou
       sn = sh + ch * th.lo;
     } else {
       k->t_stage = ts;
+      k->claim = 0;
+      k->done = 0;
     }
     k->theta2[z] = th.hi;
     k->theta2_lo[z] = th.lo;
@@ -956,6 +1001,13 @@ __global__ void k_fgeo(MeshDev md) {
   g[4 * N + j] = sgA * ag / SA;
 }
 
+// word of variable v at point j within an element face's 4 N values: variable
+// major, or in pairs of variables (ssd_stage.cuh)
+template <bool PAIRS, int N>
+__device__ __forceinline__ int face_word(int v, int j) {
+  return PAIRS ? (v >> 1) * 2 * N + 2 * j + (v & 1) : v * N + j;
+}
+
 // Conforming and periodic faces: one thread per face point; geometry from the
 // t = 0 face table, the normal turned by R(theta_z) on rotating zone z (both
 // sides of a conforming face lie in one zone).
@@ -1068,7 +1120,7 @@ __device__ __forceinline__ void bface_geom(const MeshDev &md, int b, int j, T &n
 }
 
 // Boundary faces: Rusanov through the ghost state of the face's condition.
-template <typename T, int N, bool OTF>
+template <typename T, int N, bool OTF, bool PAIRS = false>
 __device__ __forceinline__ void k_bface_point(const MeshDev &md, int t) {
   const int b = t / N, j = t - b * N;
   const int4 bf = md.bfaces[b];
@@ -1077,7 +1129,7 @@ __device__ __forceinline__ void k_bface_point(const MeshDev &md, int t) {
   const T *TR = (const T *)md.TR;
   T q[4], qg[4], qb[4];
 #pragma unroll
-  for (int v = 0; v < 4; ++v) q[v] = TR[((size_t)ef * 4 + v) * N + j];
+  for (int v = 0; v < 4; ++v) q[v] = TR[(size_t)ef * 4 * N + face_word<PAIRS, N>(v, j)];
   T nx, ny, sS, vgn, ug, vg;
   bface_geom<T, N, OTF>(md, b, j, nx, ny, sS, vgn, ug, vg);
   boundary_states(md, bf.y, q, ug, vg, nx, ny, qg, qb);
@@ -1085,7 +1137,7 @@ __device__ __forceinline__ void k_bface_point(const MeshDev &md, int t) {
   rusanov(q, qg, nx, ny, vgn, pick<T>(md.gamma, md.gamma_f), Fn);
   T *CF = (T *)md.CF;
 #pragma unroll
-  for (int v = 0; v < 4; ++v) CF[((size_t)ef * 4 + v) * N + j] = sS * Fn[v];
+  for (int v = 0; v < 4; ++v) CF[(size_t)ef * 4 * N + face_word<PAIRS, N>(v, j)] = sS * Fn[v];
 }
 
 // One launch for all face points of a stage: threads [0, nF N) take the
@@ -1096,6 +1148,15 @@ __global__ void k_faces(MeshDev md) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < md.nF * N) k_face_point<T, N, OTF>(md, t);
   else if (t < (md.nF + md.nB) * N) k_bface_point<T, N, OTF>(md, t - md.nF * N);
+}
+
+// the boundary faces alone, on traces in pairs (the stage kernel's path with
+// its phases timed apart)
+template <typename T, int N, bool OTF>
+__global__ void k_bfaces_pairs(MeshDev md) {
+  pdl_enter();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < md.nB * N) k_bface_point<T, N, OTF, true>(md, t);
 }
 
 // Mortar coupling of Sec. 3.2.  Thread (mortar, side, p): p is a quadrature
@@ -1127,20 +1188,33 @@ __device__ __forceinline__ void normal_of(double ang, T &cs, T &sn) {
   }
 }
 
-// The mortar flux of MPB mortars of block blk: thread (mortar lm < MPB, side,
-// point); threads beyond MPB * 2 N only take part in the barriers.
+// Shared memory of the mortar flux of MPB mortars.
 template <typename T, int N, int MMODE, int MPB>
-__device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk) {
-  constexpr int NV = MMODE == MORTAR_RUSANOV_FV ? 8 : 4;  // projected values per point
+struct MortShared {
+  static constexpr int NV = MMODE == MORTAR_RUSANOV_FV ? 8 : 4;  // projected values per point
   // h_i(o + s z_q) and w_q h_i(o + s z_q) [q][i]: formed in FP64, stored in
   // the compute type once
-  __shared__ T sH[MPB][2][N][N];
-  __shared__ T sWH[MPB][2][N][N];
-  __shared__ T sQf[MPB][2][NV][N];     // face values, CCW order (+ viscous normal flux)
-  __shared__ T sA[MPB][2][NV][N];      // work arrays
-  __shared__ T sB[MPB][2][NV][N];
-  __shared__ T sF[MPB][4][N];          // common mortar flux at mortar SPs
-  __shared__ T sFz[MPB][4][N];         // common flux at quadrature points
+  T H[MPB][2][N][N];
+  T WH[MPB][2][N][N];
+  T Qf[MPB][2][NV][N];  // face values, CCW order (+ viscous normal flux)
+  T A[MPB][2][NV][N];   // work arrays
+  T B[MPB][2][NV][N];
+  T F[MPB][4][N];       // common mortar flux at mortar SPs
+  T Fz[MPB][4][N];      // common flux at quadrature points
+};
+
+// The mortar flux of MPB mortars of block blk: thread (mortar lm < MPB, side,
+// point); threads beyond MPB * 2 N only take part in the barriers.
+template <typename T, int N, int MMODE, int MPB, bool PAIRS = false>
+__device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, MortShared<T, N, MMODE, MPB> &sh) {
+  constexpr int NV = MortShared<T, N, MMODE, MPB>::NV;
+  auto &sH = sh.H;
+  auto &sWH = sh.WH;
+  auto &sQf = sh.Qf;
+  auto &sA = sh.A;
+  auto &sB = sh.B;
+  auto &sF = sh.F;
+  auto &sFz = sh.Fz;
   const int lm = threadIdx.x / (2 * N);
   const int r = threadIdx.x - lm * 2 * N;
   const int sd = r / N, p = r - sd * N;
@@ -1180,7 +1254,7 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk) {
     {
       const T *TR = (const T *)md.TR;
 #pragma unroll
-      for (int v = 0; v < 4; ++v) sQf[lm][sd][v][p] = TR[((size_t)ef * 4 + v) * N + jj];
+      for (int v = 0; v < 4; ++v) sQf[lm][sd][v][p] = TR[(size_t)ef * 4 * N + face_word<PAIRS, N>(v, jj)];
     }
     // Lagrange values at the mapped quadrature point x = o + s z_p: x and its
     // distances to the SPs in FP64 (they cancel), the products in the compute
@@ -1292,10 +1366,11 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk) {
   }
 }
 
-template <typename T, int N, int MMODE>
+template <typename T, int N, int MMODE, bool PAIRS = false>
 __global__ void __launch_bounds__(MortCfg<N>::THREADS) k_mortar_flux(MeshDev md) {
   pdl_enter();
-  mortar_flux_body<T, N, MMODE, MortCfg<N>::MPB>(md, blockIdx.x);
+  __shared__ MortShared<T, N, MMODE, MortCfg<N>::MPB> sh;
+  mortar_flux_body<T, N, MMODE, MortCfg<N>::MPB, PAIRS>(md, blockIdx.x, sh);
 }
 
 // Sum of the mortar contributions of each interface face (fixed order: the
@@ -1325,6 +1400,7 @@ __device__ __forceinline__ bool gather_sum(const MeshDev &md, int fq, int p, T *
     return false;
   T acc[4] = {0, 0, 0, 0};
   int mi = start;
+#pragma unroll 1
   for (int c = 0; c < cnt; ++c) {
 #pragma unroll
     for (int v = 0; v < 4; ++v) acc[v] += cb[((size_t)mi * 4 + v) * N + p];
@@ -2160,7 +2236,8 @@ __global__ void __launch_bounds__(kFusedBlock) k_faces_mortar(MeshDev md, int nm
   pdl_enter();
   static_assert(MortCfg<N>::THREADS <= kFusedBlock, "mortar block");
   if ((int)blockIdx.x < nmb) {
-    mortar_flux_body<T, N, MMODE, MortCfg<N>::MPB>(md, blockIdx.x);
+    __shared__ MortShared<T, N, MMODE, MortCfg<N>::MPB> sh;
+    mortar_flux_body(md, blockIdx.x, sh);
     return;
   }
   const int t = ((int)blockIdx.x - nmb) * kFusedBlock + threadIdx.x;
@@ -2188,6 +2265,7 @@ static __global__ void k_advance(DevClock *clk, double dt) {
 }  // namespace ssd
 
 #include "ssd_batch.cuh"
+#include "ssd_stage.cuh"
 
 namespace ssd {
 
@@ -2229,6 +2307,24 @@ struct EngineImpl : Engine {
     if (err) return err;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, C::THREADS, C::SMEM);
   }
+  // the one-launch stage kernel (FP32 Euler)
+  template <int MODE, bool AUX>
+  static cudaError_t stage_setup(int *occ) {
+    using C = StageCfg<N, AUX, LO>;
+    auto *k = k_stage<N, MODE, AUX, LO>;
+    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    if (err) return err;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, C::THREADS, C::SMEM);
+  }
+  int early_tiles = 0;
+  int grid_st_res = 1, grid_st_rk = 1, grid_st_aux = 1;  // its persistent grid sizes
+  int stage_tile(int viscous) const override { return OTF && !viscous && !tc ? vol_epb_default<N>() : 0; }
+  void set_early_tiles(int n) override { early_tiles = n; }
+  void face_records(const MeshDev &md, const int *map, const int *row, int n, cudaStream_t s) override {
+    if constexpr (OTF)
+      k_face_records<N><<<(n + 127) / 128, 128, 0, s>>>(md, map, row, n, (float4 *)md.frec, (float4 *)md.fgp);
+  }
+
   double *dXs = nullptr, *dXf = nullptr;
   int *scratch_i = nullptr;
   double *scratch_d = nullptr;
@@ -2279,7 +2375,14 @@ struct EngineImpl : Engine {
   StatePtr A() const override { return StatePtr{sA[0], sA[1]}; }
   StatePtr B() const override { return StatePtr{sB[0], sB[1]}; }
 
-  void set_state(const MeshDev &, const double *Q, cudaStream_t s) override {
+  void set_state(const MeshDev &md, const double *Q, cudaStream_t s) override {
+    if constexpr (OTF) {
+      if (md.frec) {
+        const int n = (int)(nval / 2);
+        k_split_pairs<N * N><<<(n + 1023) / 1024, 256, 0, s>>>(Q, (float2 *)sA[0], (float2 *)sA[1], n);
+        return;
+      }
+    }
     if (DF)
       k_split<<<(unsigned)((nval + 255) / 256), 256, 0, s>>>(Q, (float *)sA[0], (float *)sA[1], nval);
     else if (OTF)
@@ -2287,7 +2390,14 @@ struct EngineImpl : Engine {
     else
       cudaMemcpyAsync(sA[0], Q, sizeof(double) * nval, cudaMemcpyDeviceToDevice, s);
   }
-  void get_state(const MeshDev &, double *Q, cudaStream_t s) override {
+  void get_state(const MeshDev &md, double *Q, cudaStream_t s) override {
+    if constexpr (OTF) {
+      if (md.frec) {
+        const int n = (int)(nval / 2);
+        k_join_pairs<N * N><<<(n + 1023) / 1024, 256, 0, s>>>((const float2 *)sA[0], (const float2 *)sA[1], Q, n);
+        return;
+      }
+    }
     if (OTF)
       k_join<<<(unsigned)((nval + 255) / 256), 256, 0, s>>>((const float *)sA[0], (const float *)sA[1], Q, nval);
     else
@@ -2355,6 +2465,15 @@ struct EngineImpl : Engine {
       if ((err = vol_setup<MODE_RESIDUAL, false, 0, One>(&occ0))) return err;
       if ((err = vol_setup<MODE_RK, false, 0, One>(&occ1))) return err;
       if ((err = vol_setup<MODE_RK, true, 0, One>(&occ2))) return err;
+      if constexpr (OTF) {
+        int o0 = 0, o1 = 0, o2 = 0;
+        if ((err = stage_setup<MODE_RESIDUAL, false>(&o0))) return err;
+        if ((err = stage_setup<MODE_RK, false>(&o1))) return err;
+        if ((err = stage_setup<MODE_RK, true>(&o2))) return err;
+        grid_st_res = std::max(1, o0) * sms;
+        grid_st_rk = std::max(1, o1) * sms;
+        grid_st_aux = std::max(1, o2) * sms;
+      }
       if constexpr (kTC) {
         int t0 = 0, t1 = 0, t2 = 0;
         if ((err = vol_setup<MODE_RESIDUAL, false, 0, One, true>(&t0))) return err;
@@ -2391,6 +2510,12 @@ struct EngineImpl : Engine {
   }
 
   void trace(const MeshDev &md, StatePtr q, cudaStream_t s) override {
+    if constexpr (OTF) {
+      if (md.frec) {
+        launch_pdl(k_trace_pairs<N>, (md.E * 8 * N + 255) / 256, 256, 0, s, md, (const float2 *)q.hi);
+        return;
+      }
+    }
     const int n = md.E * 16 * N;
     launch_pdl(k_trace<T, N>, (n + 255) / 256, 256, 0, s, md, (const T *)q.hi);
   }
@@ -2417,10 +2542,10 @@ struct EngineImpl : Engine {
   // the mortar flux as its own launch; the gather of its contributions into
   // each interface face is done by the kernel that reads the result
   // (gather_tile in k_volume, k_volume_visc, k_grad_trace)
-  template <int MMODE>
+  template <int MMODE, bool PAIRS = false>
   void mortar_flux(const MeshDev &md, cudaStream_t s) {
     constexpr int MPB = MortCfg<N>::MPB;
-    launch_pdl(k_mortar_flux<T, N, MMODE>, (md.nM + MPB - 1) / MPB, MortCfg<N>::THREADS, 0, s, md);
+    launch_pdl(k_mortar_flux<T, N, MMODE, PAIRS>, (md.nM + MPB - 1) / MPB, MortCfg<N>::THREADS, 0, s, md);
   }
 
   // a face pass fused with the mortar flux of the same pass (meshes with an
@@ -2436,6 +2561,14 @@ struct EngineImpl : Engine {
   bool fused(const MeshDev &md) const { return fuse_faces_mortar && md.nL > 0; }
 
   void faces(const MeshDev &md, StatePtr q, cudaStream_t s) override {
+    if (md.frec) {
+      // the stage kernel forms the conforming faces' fluxes itself, and the
+      // boundary points' unless the phases are timed apart
+      if (!fuse_faces_mortar && md.nB > 0) {
+        launch_pdl(k_bfaces_pairs<T, N, OTF>, (md.nB * N + 127) / 128, 128, 0, s, md);
+      }
+      return;
+    }
     const int np = (md.nF + md.nB) * N;
     if (!md.viscous) {
       if (fused(md)) fused_pass<MORTAR_RUSANOV>(md, s);
@@ -2462,8 +2595,9 @@ struct EngineImpl : Engine {
   // the mortar flux when it is not fused into the face pass (the gather is
   // done by the volume kernel)
   void mortars(const MeshDev &md, cudaStream_t s) override {
-    if (md.nL > 0 && !fused(md)) {
+    if (md.nL > 0 && !fuse_faces_mortar) {
       if (md.viscous) mortar_flux<MORTAR_RUSANOV_FV>(md, s);
+      else if (md.frec) mortar_flux<MORTAR_RUSANOV, true>(md, s);
       else mortar_flux<MORTAR_RUSANOV>(md, s);
     }
   }
@@ -2494,6 +2628,19 @@ struct EngineImpl : Engine {
                ntiles);
   }
 
+  template <int MODE, bool AUX>
+  void launch_stage(const MeshDev &md, StatePtr in, StatePtr base, StatePtr out, double *R, const RkArgs &rk, int grid,
+                    cudaStream_t s) {
+    if constexpr (OTF) {
+      using C = StageCfg<N, AUX, LO>;
+      const int ntiles = (md.E + C::EPB - 1) / C::EPB;
+      const int nmort = fuse_faces_mortar ? (md.nM + C::EPB - 1) / C::EPB : 0;
+      const int nblk = fuse_faces_mortar ? nmort + (md.nB * N + C::THREADS - 1) / C::THREADS : 0;
+      launch_pdl(k_stage<N, MODE, AUX, LO>, std::min(ntiles, grid), C::THREADS, C::SMEM, s, md,
+                 vol_args(in, base, out, R, rk), ntiles, early_tiles, nmort, nblk);
+    }
+  }
+
   void volume(const MeshDev &md, StatePtr in, StatePtr base, StatePtr out, double *R, const RkArgs &rk, int mode,
               cudaStream_t s) override {
     if (md.viscous) {
@@ -2515,6 +2662,14 @@ struct EngineImpl : Engine {
         if (mode == MODE_RESIDUAL) launch_volume<MODE_RESIDUAL, false, true>(md, in, base, out, R, rk, grid_tc_res, s);
         else if (rk.w_in) launch_volume<MODE_RK, true, true>(md, in, base, out, R, rk, grid_tc_aux, s);
         else launch_volume<MODE_RK, false, true>(md, in, base, out, R, rk, grid_tc_rk, s);
+        return;
+      }
+    }
+    if constexpr (OTF) {
+      if (md.frec) {
+        if (mode == MODE_RESIDUAL) launch_stage<MODE_RESIDUAL, false>(md, in, base, out, R, rk, grid_st_res, s);
+        else if (rk.w_in) launch_stage<MODE_RK, true>(md, in, base, out, R, rk, grid_st_aux, s);
+        else launch_stage<MODE_RK, false>(md, in, base, out, R, rk, grid_st_rk, s);
         return;
       }
     }

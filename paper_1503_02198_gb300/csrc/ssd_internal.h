@@ -41,7 +41,10 @@ struct DevClock {
   float cf[kZT], sf[kZT], omf[kZT];
   int flags;  // bit 0: non-physical state; bit 1: mesh geometry error; bit 2: a bounded device wait gave up;
               // bit 3: (debug build) a table index out of range
-  int pad;
+  // coupling blocks (mortar and boundary fluxes) of the stage kernel that reads
+  // this record: how many CTAs have claimed and how many are done; zeroed by
+  // the merge that writes the record
+  int claim, done, pad;
 };
 
 // Basis data of Sec. 3.1 and the mortar quadrature of Sec. 3.2, built on the
@@ -130,6 +133,14 @@ struct MeshDev {
   void *geo;              // T [nTab][G] metric tables (see ssd_engine.cuh)
   void *egeo;             // T [E][8] bilinear record x0, y0, e1, e3, d of each cell
   void *TR, *CF;          // T [E][4][4][N] face traces and common fluxes
+  // the traces a stage writes: TR itself where a face pass reads the old ones
+  // first, another buffer where the stage kernel reads neighbours' traces
+  // while it writes
+  void *TRo;
+  // the stage kernel's face records and per-point face table (ssd_stage.cuh),
+  // and its tiles in working order; null where it does not run
+  const float4 *frec, *fgp;
+  const int *tord;
   void *CQ, *GTR;         // viscous: T [E][4][4][N] common solution, [E][4][8][N] gradient traces
   void *GSP;              // viscous: T [E][8][N][N] gradients at the SPs (x then y, 4 variables each)
   void *fgeo;             // T [nF][5][N] conforming-face geometry at t = 0: unit normal
@@ -215,6 +226,15 @@ struct Engine {
   virtual size_t compute_word() const = 0;
   // true: straight cells get their metrics on the fly (tables only for arc cells)
   virtual bool metrics_on_the_fly() const = 0;
+  // elements per tile of the one-launch stage kernel (ssd_stage.cuh) if this
+  // engine runs it on an Euler or viscous mesh, else 0
+  virtual int stage_tile(int viscous) const = 0;
+  // that kernel's face records from the face table (map: 2 face + side or kind
+  // per element face, row: per-point table row or -1; n records, device arrays)
+  virtual void face_records(const MeshDev &md, const int *map, const int *row, int n, cudaStream_t s) = 0;
+  // the number of its tiles without an interface or boundary face (they come
+  // first in md.tord)
+  virtual void set_early_tiles(int n) = 0;
   // get / set the tunable launch shapes (see EngineImpl::tuning)
   virtual void tuning(int *vol_ctas_per_sm, int *max_ctas_per_sm, int *face_block) = 0;
   // the two state buffers A and B: E elements, storage for Epad >= E
