@@ -198,9 +198,7 @@ struct sd_handle {
   // (the last captured step has merged them)
   bool tables_valid = false;
   double tables_dt = 0.0;
-  // per element face: 2 face + side, or the kind of a face that is not a
-  // conforming one (see ssd_stage.cuh)
-  std::vector<int> efmap;
+  std::vector<int> bface_v;  // element faces of the boundary
   bool in_batch = false;  // a batch's case: its kernels are the batch's (state and traces one variable at a time)
   // the captured step, one per set of stage tables it reads (see queue_step)
   cudaGraphExec_t step_exec[2] = {nullptr, nullptr};
@@ -504,12 +502,7 @@ int build_mesh(sd_handle *h, const sd_mesh *m, double omega1) {
   h->iface_v.assign(E, 0);
   for (int ef = 0; ef < 4 * E; ++ef)
     if (efi[ef] >= 0) h->iface_v[ef / 4] = 1;
-  h->efmap.assign(4 * (size_t)E, -1);
-  for (size_t k = 0; k < faces.size(); ++k) {
-    h->efmap[faces[k].x] = (int)(2 * k);
-    h->efmap[faces[k].y] = (int)(2 * k + 1);
-  }
-  for (const int4 &b : bfaces) h->efmap[b.x] = -2;
+  for (const int4 &b : bfaces) h->bface_v.push_back(b.x);
   cudaError_t ce;
   int4 *dfaces, *dbfaces, *dL, *dR;
   double *dcorn, *dLa, *dLw, *dLS, *dRa, *dRw, *dRS, *dLiW, *dRiW, *dcub = nullptr, *dzpar, *dLal, *dRal;
@@ -599,8 +592,9 @@ cudaError_t alloc_buffers(sd_handle *h, const std::vector<int> &zone, const std:
     // tiles in working order: those with an interface or boundary face last
     const int nt = (int)((E + epb - 1) / epb);
     std::vector<char> late(nt, 0);
-    for (size_t ef = 0; ef < 4 * E; ++ef)
-      if (h->efmap[ef] < 0) late[ef / 4 / epb] = 1;
+    for (size_t k = 0; k < E; ++k)
+      if (h->iface_v[k]) late[k / epb] = 1;
+    for (int ef : h->bface_v) late[ef / 4 / epb] = 1;
     std::vector<int> order;
     for (int pass = 0; pass < 2; ++pass) {
       for (int t = 0; t < nt; ++t)
@@ -678,35 +672,26 @@ cudaError_t alloc_buffers(sd_handle *h, const std::vector<int> &zone, const std:
   return cudaStreamSynchronize(h->stream);
 }
 
-// The stage kernel's face records (after the engine has formed the face
-// table).  A face needs its own per-point row where the normal or V_g.n varies
-// along it: on rotating zones and next to curved cells.
+// The stage kernel's face records (after the engine has formed the face table)
 cudaError_t build_face_records(sd_handle *h) {
   MeshDev &md = h->md;
-  if (h->in_batch || !h->eng->stage_tile(md.viscous)) return cudaSuccess;
-  const size_t E = md.E, N = h->N, Ep = (E + kElemPad - 1) / kElemPad * kElemPad;
-  std::vector<char> varies(md.nF ? md.nF : 1, 0);
-  for (size_t ef = 0; ef < 4 * E; ++ef)
-    if (h->efmap[ef] >= 0 && (h->zone_v[ef / 4] || h->curved_v[ef / 4])) varies[h->efmap[ef] >> 1] = 1;
-  std::vector<int> row(4 * Ep, -1);
-  int rows = 0;
-  for (size_t ef = 0; ef < 4 * E; ++ef)
-    if (h->efmap[ef] >= 0 && varies[h->efmap[ef] >> 1]) row[ef] = rows++;
+  if (!md.tord) return cudaSuccess;
+  const size_t N = h->N, Ep = ((size_t)md.E + kElemPad - 1) / kElemPad * kElemPad;
+  int *hp = (int *)h->h_pinned, *count = &md.clk->claim;  // (a counter that is 0 until the first merge, and zeroed by it)
   float4 *rec, *pts;
-  int *tmp = nullptr;
   cudaError_t e;
+  h->eng->face_records(md, nullptr, nullptr, count, h->stream);
+  if ((e = cudaMemcpyAsync(hp, count, sizeof(int), cudaMemcpyDeviceToHost, h->stream))) return e;
+  if ((e = cudaMemsetAsync(count, 0, sizeof(int), h->stream))) return e;
+  if ((e = cudaStreamSynchronize(h->stream))) return e;
   if ((e = dalloc(h, &rec, sizeof(float4) * 4 * Ep))) return e;
-  if ((e = dalloc(h, &pts, sizeof(float4) * N * rows))) return e;
+  if ((e = dalloc(h, &pts, sizeof(float4) * 2 * N * (size_t)*hp))) return e;
+  if ((e = cudaMemsetAsync(rec, 0, sizeof(float4) * 4 * Ep, h->stream))) return e;
   md.frec = rec;
   md.fgp = pts;
-  if ((e = cudaMalloc(&tmp, sizeof(int) * 8 * Ep))) return e;
-  e = cudaMemcpyAsync(tmp, h->efmap.data(), sizeof(int) * 4 * E, cudaMemcpyHostToDevice, h->stream);
-  if (!e) e = cudaMemcpyAsync(tmp + 4 * Ep, row.data(), sizeof(int) * 4 * Ep, cudaMemcpyHostToDevice, h->stream);
-  if (!e) h->eng->face_records(md, tmp, tmp + 4 * Ep, (int)(4 * Ep), h->stream);
-  if (!e) e = cudaGetLastError();
-  if (!e) e = cudaStreamSynchronize(h->stream);
-  cudaFree(tmp);
-  return e;
+  h->eng->face_records(md, rec, pts, count, h->stream);
+  if ((e = cudaMemsetAsync(count, 0, sizeof(int), h->stream))) return e;
+  return cudaGetLastError();
 }
 
 // device flags: the OR of the primary clock's and the stage records' of both
@@ -922,7 +907,9 @@ void queue_step(sd_handle *h, double dt, int ts) {
   h->eng->merge_stages(h->md, ts ? h->sm : h->sm_b, dt, 0, n, 1, kSideMergeThreads, h->side);
   h->eng->advance(h->md, dt, h->side);
   cudaEventRecord(h->ev_next, h->side);
+  h->eng->set_tables_ready(true);  // merged beside the step before
   for (int k = 0; k < n; ++k) queue_stage(h, plan[k].md, plan[k].in, plan[k].base, plan[k].out, plan[k].rk);
+  h->eng->set_tables_ready(false);
   cudaStreamWaitEvent(h->stream, h->ev_next, 0);
 }
 

@@ -58,6 +58,17 @@ namespace ssd {
 // waits for its predecessor before it can complete, the order of the whole
 // stream is kept.
 __device__ __forceinline__ void pdl_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The stage kernel's launches in a captured step may do better.  ahead 0: wait
+// at once.  ahead 1: the stage's tables (clock, mortar table, Eq. xz) and the mesh were
+// complete before the step began, so a block reads them first and waits where
+// it first touches the flow (pdl_enter there; a second wait returns at once).
+// ahead 2: the grid also lets the next launch's blocks in as soon as its own
+// are all running, to do the same beside it; only for short grids, where the
+// parked blocks' slots are not missed and the launch latency is.
+__device__ __forceinline__ void pdl_begin(int ahead) {
+  if (ahead == 2) asm volatile("griddepcontrol.launch_dependents;");
+  if (ahead == 0) pdl_enter();
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
@@ -1201,12 +1212,22 @@ struct MortShared {
   T B[MPB][2][NV][N];
   T F[MPB][4][N];       // common mortar flux at mortar SPs
   T Fz[MPB][4][N];      // common flux at quadrature points
+  // h_j(z_q), w_q h_j(z_q) and M^{-1}: a warp's threads read different rows,
+  // which constant memory would serve one at a time
+  T Hz[N * N], wHz[N * N], Mi[N * N];
 };
 
 // The mortar flux of MPB mortars of block blk: thread (mortar lm < MPB, side,
 // point); threads beyond MPB * 2 N only take part in the barriers.
-template <typename T, int N, int MMODE, int MPB, bool PAIRS = false>
-__device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, MortShared<T, N, MMODE, MPB> &sh) {
+// enter() is called between the part that reads the stage's tables only and the
+// part that reads the flow (a kernel that starts ahead of its predecessor's end
+// waits for it there).
+struct NoWait {
+  __device__ __forceinline__ void operator()() const {}
+};
+template <typename T, int N, int MMODE, int MPB, bool PAIRS = false, class Enter = NoWait>
+__device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, MortShared<T, N, MMODE, MPB> &sh,
+                                                 Enter enter = Enter()) {
   constexpr int NV = MortShared<T, N, MMODE, MPB>::NV;
   auto &sH = sh.H;
   auto &sWH = sh.WH;
@@ -1223,18 +1244,10 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
   const MortBasis<N> &B = cMB<N>;
   double o = 0.0, s = 0.0;
   int ef = 0, rev = 0;
-  double m0 = 0.0, dm = 0.0;
-  if (act) {
-    // Eq. xz: offset and scale of this mortar against its face on side sd,
-    // formed by the stage's merge
-    const MortSide ms = md.msd[(size_t)sd * md.nM + m];
-    m0 = md.mgeo[4 * m];
-    dm = md.mgeo[4 * m + 2];
-    o = ms.o;
-    s = ms.s;
-    ef = ms.ef;
-    rev = ms.rev;
-    if (!ssd_check(md, ef >= 0 && ef < 4 * md.E)) ef = 0;
+  T mcs = 0, msn = 0, fcs = 0, fsn = 0;  // radial normals at mortar SP p and at face point p
+  constexpr bool kDefer = !std::is_same<Enter, NoWait>::value;
+  // this point's flow data, in counter-clockwise point order
+  auto load_flow = [&]() {
     const int jj = rev ? N - 1 - p : p;
     if (MMODE == MORTAR_RUSANOV_FV) {
       // viscous normal flux of this face point with the common solution and
@@ -1245,9 +1258,7 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
       for (int v = 0; v < 4; ++v) q[v] = CQ[((size_t)ef * 4 + v) * N + jj];
 #pragma unroll
       for (int c = 0; c < 8; ++c) g8[c] = GT[((size_t)ef * 8 + c) * N + jj];
-      T sn, cs;
-      normal_of<T>(ms.fa_hi + (ms.fa_lo + B.Xs[p] * ms.w), cs, sn);
-      viscous_normal(q, g8, cs, sn, md, fn);
+      viscous_normal(q, g8, fcs, fsn, md, fn);
 #pragma unroll
       for (int v = 0; v < 4; ++v) sQf[lm][sd][NV - 4 + v][p] = fn[v];
     }
@@ -1256,6 +1267,25 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
 #pragma unroll
       for (int v = 0; v < 4; ++v) sQf[lm][sd][v][p] = TR[(size_t)ef * 4 * N + face_word<PAIRS, N>(v, jj)];
     }
+  };
+  for (int k = threadIdx.x; k < N * N; k += blockDim.x) {
+    sh.Hz[k] = pick<T>(B.Hz[k], B.Hz_f[k]);
+    sh.wHz[k] = pick<T>(B.wHz[k], B.wHz_f[k]);
+    sh.Mi[k] = pick<T>(B.Minv[k], B.Minv_f[k]);
+  }
+  if (act) {
+    // Eq. xz: offset and scale of this mortar against its face on side sd,
+    // formed by the stage's merge
+    const MortSide ms = md.msd[(size_t)sd * md.nM + m];
+    const double m0 = md.mgeo[4 * m], m0_lo = md.mgeo[4 * m + 1], dm = md.mgeo[4 * m + 2];
+    o = ms.o;
+    s = ms.s;
+    ef = ms.ef;
+    rev = ms.rev;
+    if (!ssd_check(md, ef >= 0 && ef < 4 * md.E)) ef = 0;
+    if (MMODE == MORTAR_RUSANOV_FV) normal_of<T>(ms.fa_hi + (ms.fa_lo + B.Xs[p] * ms.w), fcs, fsn);
+    if constexpr (!kDefer) load_flow();
+    if (MMODE != MORTAR_AVG_Q && sd == 0) normal_of<T>(m0 + fma(B.Xs[p], dm, m0_lo), mcs, msn);
     // Lagrange values at the mapped quadrature point x = o + s z_p: x and its
     // distances to the SPs in FP64 (they cancel), the products in the compute
     // type (on the FP32 path each weight is then good to a few float ulps)
@@ -1272,6 +1302,10 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
       sH[lm][sd][p][i] = h;
       sWH[lm][sd][p][i] = (T)B.wq[p] * h;
     }
+  }
+  if constexpr (kDefer) {
+    enter();
+    if (act) load_flow();
   }
   __syncthreads();
   // (A) face polynomial at the mapped quadrature points
@@ -1291,7 +1325,7 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
     for (int v = 0; v < NV; ++v) {
       T acc = 0;
 #pragma unroll
-      for (int q = 0; q < N; ++q) acc += pick<T>(B.wHz[q * N + p], B.wHz_f[q * N + p]) * sA[lm][sd][v][q];
+      for (int q = 0; q < N; ++q) acc += sh.wHz[q * N + p] * sA[lm][sd][v][q];
       sB[lm][sd][v][p] = acc;
     }
   }
@@ -1302,7 +1336,7 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
     for (int v = 0; v < NV; ++v) {
       T acc = 0;
 #pragma unroll
-      for (int k = 0; k < N; ++k) acc += pick<T>(B.Minv[p * N + k], B.Minv_f[p * N + k]) * sB[lm][sd][v][k];
+      for (int k = 0; k < N; ++k) acc += sh.Mi[p * N + k] * sB[lm][sd][v][k];
       sA[lm][sd][v][p] = acc;
     }
   }
@@ -1311,15 +1345,13 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
   // a rotation about the circle's centre is tangential: v_g . n = 0)
   if (act && sd == 0) {
     if (MMODE != MORTAR_AVG_Q) {
-      T sn, cs;
-      normal_of<T>(m0 + fma(B.Xs[p], dm, md.mgeo[4 * m + 1]), cs, sn);
       T qL[4], qR[4], Fn[4];
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         qL[v] = sA[lm][0][v][p];
         qR[v] = sA[lm][1][v][p];
       }
-      rusanov(qL, qR, (T)cs, (T)sn, T(0), pick<T>(md.gamma, md.gamma_f), Fn);
+      rusanov(qL, qR, mcs, msn, T(0), pick<T>(md.gamma, md.gamma_f), Fn);
 #pragma unroll
       for (int v = 0; v < 4; ++v)
         sF[lm][v][p] = MMODE == MORTAR_RUSANOV_FV ? Fn[v] + T(0.5) * (sA[lm][0][4 + v][p] + sA[lm][1][4 + v][p])
@@ -1337,7 +1369,7 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
     for (int v = 0; v < 4; ++v) {
       T acc = 0;
 #pragma unroll
-      for (int j = 0; j < N; ++j) acc += pick<T>(B.Hz[p * N + j], B.Hz_f[p * N + j]) * sF[lm][v][j];
+      for (int j = 0; j < N; ++j) acc += sh.Hz[p * N + j] * sF[lm][v][j];
       sFz[lm][v][p] = acc;
     }
   }
@@ -1360,7 +1392,7 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
     for (int v = 0; v < 4; ++v) {
       T acc = 0;
 #pragma unroll
-      for (int k = 0; k < N; ++k) acc += pick<T>(B.Minv[p * N + k], B.Minv_f[p * N + k]) * sB[lm][sd][v][k];
+      for (int k = 0; k < N; ++k) acc += sh.Mi[p * N + k] * sB[lm][sd][v][k];
       out[v * N + p] = (T)s * acc;
     }
   }
@@ -2237,7 +2269,7 @@ __global__ void __launch_bounds__(kFusedBlock) k_faces_mortar(MeshDev md, int nm
   static_assert(MortCfg<N>::THREADS <= kFusedBlock, "mortar block");
   if ((int)blockIdx.x < nmb) {
     __shared__ MortShared<T, N, MMODE, MortCfg<N>::MPB> sh;
-    mortar_flux_body(md, blockIdx.x, sh);
+    mortar_flux_body<T, N, MMODE, MortCfg<N>::MPB>(md, blockIdx.x, sh);
     return;
   }
   const int t = ((int)blockIdx.x - nmb) * kFusedBlock + threadIdx.x;
@@ -2320,9 +2352,10 @@ struct EngineImpl : Engine {
   int grid_st_res = 1, grid_st_rk = 1, grid_st_aux = 1;  // its persistent grid sizes
   int stage_tile(int viscous) const override { return OTF && !viscous && !tc ? vol_epb_default<N>() : 0; }
   void set_early_tiles(int n) override { early_tiles = n; }
-  void face_records(const MeshDev &md, const int *map, const int *row, int n, cudaStream_t s) override {
+  void face_records(const MeshDev &md, float4 *rec, float4 *pts, int *count, cudaStream_t s) override {
+    const int n = md.nF + md.nL + md.nR + md.nB;
     if constexpr (OTF)
-      k_face_records<N><<<(n + 127) / 128, 128, 0, s>>>(md, map, row, n, (float4 *)md.frec, (float4 *)md.fgp);
+      if (n > 0) k_face_records<N><<<(n + 127) / 128, 128, 0, s>>>(md, rec, pts, count);
   }
 
   double *dXs = nullptr, *dXf = nullptr;
@@ -2558,6 +2591,16 @@ struct EngineImpl : Engine {
     launch_pdl(k_faces_mortar<T, N, OTF, MMODE>, nmb + (np + kFusedBlock - 1) / kFusedBlock, kFusedBlock, 0, s, md,
                nmb);
   }
+  // How far a launch of a captured step may run ahead (pdl_begin).  The stage
+  // kernel lets its successor in while its grid has at most four tiles per
+  // block: 33.5 -> 29.0 us a step on 6,016 cells at N = 4, 43.3 -> 32.3 at N = 5,
+  // 52.7 -> 51.5 on 31,509 cells at N = 3 (2.6 tiles per block), but 605 -> 611 on
+  // 246,900 cells (41 tiles).  The launches of a viscous stage wait at once (four
+  // different kernels: parked blocks settle unevenly beside the running ones;
+  // 14,752 cells 193 -> 223 us a step, 20,096 cells 181 -> 200).
+  bool tables_ready = false;
+  void set_tables_ready(bool on) override { tables_ready = on; }
+  int ahead_stage(int tiles, int grid) const { return tables_ready ? (tiles <= 4 * grid ? 2 : 1) : 0; }
   bool fused(const MeshDev &md) const { return fuse_faces_mortar && md.nL > 0; }
 
   void faces(const MeshDev &md, StatePtr q, cudaStream_t s) override {
@@ -2636,8 +2679,8 @@ struct EngineImpl : Engine {
       const int ntiles = (md.E + C::EPB - 1) / C::EPB;
       const int nmort = fuse_faces_mortar ? (md.nM + C::EPB - 1) / C::EPB : 0;
       const int nblk = fuse_faces_mortar ? nmort + (md.nB * N + C::THREADS - 1) / C::THREADS : 0;
-      launch_pdl(k_stage<N, MODE, AUX, LO>, std::min(ntiles, grid), C::THREADS, C::SMEM, s, md,
-                 vol_args(in, base, out, R, rk), ntiles, early_tiles, nmort, nblk);
+      launch_pdl(k_stage<N, MODE, AUX, LO>, std::min(ntiles, grid), C::THREADS, C::SMEM, s, md, vol_args(in, base, out, R, rk), ntiles,
+                 early_tiles, nmort, nblk, ahead_stage(ntiles, grid));
     }
   }
 

@@ -229,9 +229,10 @@ struct Engine {
   // elements per tile of the one-launch stage kernel (ssd_stage.cuh) if this
   // engine runs it on an Euler or viscous mesh, else 0
   virtual int stage_tile(int viscous) const = 0;
-  // that kernel's face records from the face table (map: 2 face + side or kind
-  // per element face, row: per-point table row or -1; n records, device arrays)
-  virtual void face_records(const MeshDev &md, const int *map, const int *row, int n, cudaStream_t s) = 0;
+  // that kernel's face records rec (zeroed by the caller) and per-point rows pts
+  // from the face table; with rec null only *count, the number of faces with two
+  // such rows (*count: device memory, 0 before)
+  virtual void face_records(const MeshDev &md, float4 *rec, float4 *pts, int *count, cudaStream_t s) = 0;
   // the number of its tiles without an interface or boundary face (they come
   // first in md.tord)
   virtual void set_early_tiles(int n) = 0;
@@ -267,6 +268,10 @@ struct Engine {
   // true (default): the mortar flux runs inside the face launch of the same
   // pass; false: as its own launch in mortars() (per-phase timing)
   virtual void set_fusion(bool on) = 0;
+  // the launches that follow belong to a captured step: its tables (clocks,
+  // mortar tables, Eq. xz) were complete before the step began, so a kernel may
+  // read them before the launch ahead of it has ended
+  virtual void set_tables_ready(bool on) = 0;
   // the inviscid volume kernel's interpolation and divergence contractions on
   // the tensor cores (3xTF32; FP32 form only); returns false if unavailable
   virtual bool set_tensor_cores(bool on) = 0;

@@ -126,38 +126,46 @@ __global__ void k_trace_pairs(MeshDev md, const float2 *__restrict__ Q) {
 // branch).
 constexpr float kRecTable = 2.0f, kRecIface = 3.0f, kRecBoundary = 4.0f;
 
-// records of every element face from the face table (one thread per element
-// face); map[ef] = 2 face + side or a kind, row[ef] = row of the per-point
-// table or -1
+// The records from the face table: one thread per conforming or periodic face
+// (its two element faces), then per interface and boundary face.  With rec
+// null only the faces that need per-point rows are counted; else each of them
+// takes its next two rows of pts from the counter.
 template <int N>
-__global__ void k_face_records(MeshDev md, const int *__restrict__ map, const int *__restrict__ row, int n,
-                               float4 *rec, float4 *pts) {
-  const int ef = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ef >= n) return;
-  float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);  // padding: reads the first face's traces, is not used
-  const int m = ef < 4 * md.E ? map[ef] : 0;
-  if (ef < 4 * md.E && m < 0) {
-    r.x = m == -1 ? kRecIface : kRecBoundary;
-    r.w = __int_as_float(ef * 4 * N);
-  } else if (ef < 4 * md.E) {
-    const int fi = m >> 1, side = m & 1;
-    const int4 fc = md.faces[fi];
-    const float *g = (const float *)md.fgeo + (size_t)fi * 5 * N;
-    r.w = __int_as_float((side ? fc.x : fc.y) * 4 * N | (fc.z ? 2 : 0) | side);
-    if (row[ef] < 0) {
-      r.x = g[0];
-      r.y = g[N];
-      r.z = side ? -g[3 * N] : g[2 * N];
-    } else {
-      r.x = kRecTable;
-      r.y = __int_as_float(row[ef]);
-      for (int p = 0; p < N; ++p) {
-        const int j = (side && fc.z) ? N - 1 - p : p;  // the table is in side A's point order
-        pts[(size_t)row[ef] * N + p] = make_float4(g[j], g[N + j], side ? -g[3 * N + j] : g[2 * N + j], g[4 * N + j]);
+__global__ void k_face_records(MeshDev md, float4 *rec, float4 *pts, int *count) {
+  int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < md.nF) {
+    const int4 fc = md.faces[t];
+    // the normal or V_g.n varies along the face on rotating zones (low bits of
+    // the cell flag) and next to cells with a metric table
+    const bool varies = ((md.eflag[fc.x >> 2] | md.eflag[fc.y >> 2]) & ~kIfaceBit) != 0;
+    const int row = varies ? 2 * atomicAdd(count, 1) : 0;
+    if (!rec) return;
+    const float *g = (const float *)md.fgeo + (size_t)t * 5 * N;
+    for (int side = 0; side < 2; ++side) {
+      float4 r;
+      r.w = __int_as_float((side ? fc.x : fc.y) * 4 * N | (fc.z ? 2 : 0) | side);
+      if (!varies) {
+        r.x = g[0];
+        r.y = g[N];
+        r.z = side ? -g[3 * N] : g[2 * N];
+      } else {
+        r.x = kRecTable;
+        r.y = __int_as_float(row + side);
+        r.z = 0.0f;
+        for (int p = 0; p < N; ++p) {
+          const int j = (side && fc.z) ? N - 1 - p : p;  // the table is in side A's point order
+          pts[(size_t)(row + side) * N + p] = make_float4(g[j], g[N + j], side ? -g[3 * N + j] : g[2 * N + j], g[4 * N + j]);
+        }
       }
+      rec[side ? fc.y : fc.x] = r;
     }
+    return;
   }
-  rec[ef] = r;
+  t -= md.nF;
+  if (!rec || t >= md.nL + md.nR + md.nB) return;
+  const bool iface = t < md.nL + md.nR;
+  const int ef = t < md.nL ? md.Lface[t].x : iface ? md.Rface[t - md.nL].x : md.bfaces[t - md.nL - md.nR].x;
+  rec[ef] = make_float4(iface ? kRecIface : kRecBoundary, 0.0f, 0.0f, __int_as_float(ef * 4 * N));
 }
 
 // Rusanov common fluxes (Sec. 3.1) of a line's two end points, one per lane:
@@ -272,8 +280,8 @@ __device__ __forceinline__ bool wait_coupling(const int *done, int nblk) {
 template <int N, int MODE, bool AUX, bool LO>
 __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX, LO>::MINB)
     k_stage(const __grid_constant__ MeshDev md, const __grid_constant__ VolArgs<float> va, int nitems, int nearly,
-            int nmort, int nblk) {
-  pdl_enter();
+            int nmort, int nblk, int ahead) {
+  pdl_begin(ahead);
   using C = StageCfg<N, AUX, LO>;
   constexpr int EPB = C::EPB, NT = C::THREADS, NN = N * N;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -295,21 +303,21 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
   // first tile brings its own face records too (slot 0).  (The test switch of
   // sd_test_wait_timeout arms the first tile of CTA 0 with more bytes than its
   // copies deliver; it is 0 otherwise.)
-  auto issueA = [&](int tile, int st, int tile2, int slot2, bool first, int lane) {
+  auto issue_tables = [&](int tile, int st, int tile2, int slot2, bool first) {
     unsigned char *sb = smem + st * C::STAGE;
     const size_t e0 = (size_t)tile * EPB;
-    if (lane == 0)
-      mbar_expect_tx(&bar[st], C::TXA + (tile2 >= 0 ? C::RECB : 0) +
-                                   (first ? C::RECB + (blockIdx.x == 0 ? md.test_tx_extra : 0) : 0));
-    __syncwarp();
+    mbar_expect_tx(&bar[st], C::TXA + (tile2 >= 0 ? C::RECB : 0) +
+                                 (first ? C::RECB + (blockIdx.x == 0 ? md.test_tx_extra : 0) : 0));
+    bulk_g2s(sb + C::O_EG, (const float *)md.egeo + e0 * 8, C::EGB, &bar[st]);
+    bulk_g2s(sb + C::O_EF, md.eflag + e0, C::EFB, &bar[st]);
+    if (first) issue_rec(tile, 0, &bar[st]);
+    if (tile2 >= 0) issue_rec(tile2, slot2, &bar[st]);
+  };
+  // (after issue_tables has armed the barrier)
+  auto issue_state = [&](int tile, int st, int lane) {
     if (lane < EPB)
-      bulk_g2s(sb + C::O_QHI + lane * C::SE * 4, (const float *)va.in.hi + (e0 + lane) * 4 * NN, C::QE, &bar[st]);
-    if (lane == 0) {
-      bulk_g2s(sb + C::O_EG, (const float *)md.egeo + e0 * 8, C::EGB, &bar[st]);
-      bulk_g2s(sb + C::O_EF, md.eflag + e0, C::EFB, &bar[st]);
-      if (first) issue_rec(tile, 0, &bar[st]);
-      if (tile2 >= 0) issue_rec(tile2, slot2, &bar[st]);
-    }
+      bulk_g2s(smem + st * C::STAGE + C::O_QHI + lane * C::SE * 4,
+               (const float *)va.in.hi + ((size_t)tile * EPB + lane) * 4 * NN, C::QE, &bar[st]);
   };
   auto issueB = [&](int tile) {
     const size_t e0 = (size_t)tile * EPB;
@@ -322,10 +330,16 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
     if (AUX) bulk_g2s(smem + C::O_AUX, va.w_in + e0 * 4 * NN, C::AUXB, &bar[2]);
   };
   // one coupling block: EPB mortars, or NT boundary points
+  bool entered = ahead == 0;
+  auto enter = [&]() {  // what the launch before this one wrote may be read from here on
+    if (!entered) pdl_enter();
+    entered = true;
+  };
   auto couple = [&](int c) {
     if (c < nmort) {
-      mortar_flux_body<float, N, MORTAR_RUSANOV, EPB, true>(md, c, *(typename C::Mort *)(smem + C::O_QLO));
+      mortar_flux_body<float, N, MORTAR_RUSANOV, EPB, true>(md, c, *(typename C::Mort *)(smem + C::O_QLO), enter);
     } else {
+      enter();
       const int t = (c - nmort) * NT + threadIdx.x;
       if (t < md.nB * N) k_bface_point<float, N, true, true>(md, t);
     }
@@ -356,13 +370,19 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
   int tile1 = item + G < nitems ? md.tord[item + G] : -1;
   int tile2 = item + 2 * G < nitems ? md.tord[item + 2 * G] : -1;
   __syncthreads();
-  if (threadIdx.x < 32 && tile >= 0) issueA(tile, 0, tile1, 1, true, threadIdx.x);
-  // the first CTAs take the coupling blocks before their tiles
-  if ((int)blockIdx.x < nblk) {
+  if (threadIdx.x == 0 && tile >= 0) issue_tables(tile, 0, tile1, 1, true);
+  // the first CTAs take the coupling blocks before their tiles, and so does a
+  // CTA whose first tile needs them, as long as any is unclaimed
+  bool claimed = nblk == 0;  // every block has been claimed
+  if ((int)blockIdx.x < nblk || (item >= nearly && !claimed)) {
     const int c = claim();
     if (c < nblk) couple(c);
+    else claimed = true;
   }
   bool ready = nblk == 0;
+  enter();
+  __syncwarp();
+  if (threadIdx.x < 32 && tile >= 0) issue_state(tile, 0, threadIdx.x);
 
   // this thread's SP line (direction d: 0 xi, 1 eta) and its two end faces
   const int d = threadIdx.x >= EPB * N ? 1 : 0;
@@ -429,20 +449,16 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
       // the refilled regions were last read before the previous iteration's
       // closing barrier; order those generic reads before the async writes
       fence_proxy_async_smem();
-      issueA(tile1, st ^ 1, tile2, slot2, false, threadIdx.x);
+      if (threadIdx.x == 0) issue_tables(tile1, st ^ 1, tile2, slot2, false);
+      __syncwarp();
+      issue_state(tile1, st ^ 1, threadIdx.x);
     }
-    if (!ready && item >= nearly) {
-      // this tile needs the coupling blocks' results: a block left unclaimed
-      // is taken here (before the Runge-Kutta inputs fill the region its work
-      // arrays lie over); then every block has been claimed by a running CTA
+    if (!claimed && item >= nearly) {
+      // this tile needs the coupling blocks' results: a block left unclaimed is
+      // taken here (before the Runge-Kutta inputs fill the region its work
+      // arrays lie over), so that each one is in the hands of a running CTA
       for (int c = claim(); c < nblk; c = claim()) couple(c);
-      bool done = true;
-      if (threadIdx.x == 0) done = wait_coupling(&md.clk->done, nblk);
-      if (!__syncthreads_and(done)) {
-        give_up(it, true, false);
-        return;
-      }
-      ready = true;
+      claimed = true;
     }
     if (txB && threadIdx.x == 0) {
       fence_proxy_async_smem();
@@ -475,6 +491,7 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
       if (moving) Gm.load_rec(md, e0 + le, sEF[le], sEG + le * 8, sZT);
       else Gm.load_still(md, sEF[le], sEG + le * 8);
       float2 f01[N + 1], f23[N + 1];
+      float2 kind;  // above kRecTable: not a conforming face
       {
         // own traces (as the trace phase formed them), then the Rusanov fluxes
         // of both ends, one per lane; on rotating zones the normal is turned
@@ -513,19 +530,7 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
         }
 #pragma unroll
         for (int v = 0; v < 4; ++v) F[v] = f2_mul(fs, F[v]);
-        if (le < ne && fmaxf(nx.x, nx.y) > kRecTable) {
-          float val[4];
-          if (nx.x > kRecTable) {
-            special(4 * (e0 + le) + fa, nx.x, val);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) F[v].x = val[v];
-          }
-          if (nx.y > kRecTable) {
-            special(4 * (e0 + le) + fb, nx.y, val);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) F[v].y = val[v];
-          }
-        }
+        kind = make_float2(nx.x, nx.y);
         f01[0] = make_float2(F[0].x, F[1].x);
         f23[0] = make_float2(F[2].x, F[3].x);
         f01[N] = make_float2(F[0].y, F[1].y);
@@ -579,6 +584,32 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
           point_flux_still(qf, mvx[i], mvy[i], gm1, f);
           f01[i] = make_float2(f[0], f[1]);
           f23[i] = make_float2(f[2], f[3]);
+        }
+      }
+      if (item >= nearly) {
+        // the end points that are not conforming ones, once the coupling blocks
+        // are done
+        if (!ready) {
+          bool done = true;
+          if (threadIdx.x == 0) done = wait_coupling(&md.clk->done, nblk);
+          if (!__syncthreads_and(done)) {
+            give_up(it, false, txB != 0);
+            return;
+          }
+          ready = true;
+        }
+        if (le < ne) {
+          float val[4];
+          if (kind.x > kRecTable) {
+            special(4 * (e0 + le) + fa, kind.x, val);
+            f01[0] = make_float2(val[0], val[1]);
+            f23[0] = make_float2(val[2], val[3]);
+          }
+          if (kind.y > kRecTable) {
+            special(4 * (e0 + le) + fb, kind.y, val);
+            f01[N] = make_float2(val[0], val[1]);
+            f23[N] = make_float2(val[2], val[3]);
+          }
         }
       }
       float2 acc0[N], acc1[N];
