@@ -184,7 +184,7 @@ struct sd_handle {
   MeshDev md{};
   std::vector<void *> allocs;
   std::vector<int> zone_v, curved_v, iface_v;  // per element: zone, has an arc edge, has an interface face
-  double *stage = nullptr;    // FP64 staging of host states (FP32 path)
+  double *stage = nullptr;    // FP64 staging of host states (where the engine converts them)
   double *scratch = nullptr;  // device copy of a host residual
   // the face-trace buffers; two where the stage kernel reads one and writes the
   // other, else the same one twice
@@ -578,7 +578,7 @@ cudaError_t alloc_buffers(sd_handle *h, const std::vector<int> &zone, const std:
   md.tab_elem = dtab;
   md.nTab = (int)tab_elem.size();
   if ((e = h->eng->alloc_state((int)E, (int)Ep))) return e;
-  if (otf && (e = dalloc(h, &h->stage, sizeof(double) * E * 4 * N * N))) return e;
+  if ((otf || md.viscous) && (e = dalloc(h, &h->stage, sizeof(double) * E * 4 * N * N))) return e;
   if ((e = dalloc(h, &md.geo, w * (tab_elem.size() ? tab_elem.size() : 1) * h->eng->geo_words()))) return e;
   md.egeo = nullptr;
   if (otf && (e = dalloc(h, &md.egeo, w * Ep * 8))) return e;
@@ -1054,6 +1054,8 @@ int sd_info(const sd_handle *h, int *n_elems, int *N, long long *n_dofs) {
   return SD_OK;
 }
 
+// the engine holds the state in another form than the ABI's [E][4][N][N] doubles
+static bool converted_state(const sd_handle *h) { return h->eng->metrics_on_the_fly() || h->md.viscous; }
 static size_t state_bytes(const sd_handle *h) { return sizeof(double) * (size_t)h->E * 4 * h->N * h->N; }
 
 }  // extern "C"
@@ -1078,7 +1080,7 @@ extern "C" {
 int sd_set_state(sd_handle *h, const double *Q, int on_device) {
   if (!h || !Q) return fail(h, SD_ERR_ARG, "null argument");
   cudaError_t e = cudaSuccess;
-  if (!h->eng->metrics_on_the_fly()) {
+  if (!converted_state(h)) {
     e = cudaMemcpyAsync(h->eng->A().hi, Q, state_bytes(h),
                         on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream);
   } else {
@@ -1101,7 +1103,7 @@ int sd_set_state(sd_handle *h, const double *Q, int on_device) {
 int sd_get_state(sd_handle *h, double *Q, int on_device) {
   if (!h || !Q) return fail(h, SD_ERR_ARG, "null argument");
   cudaError_t e = cudaSuccess;
-  if (!h->eng->metrics_on_the_fly()) {
+  if (!converted_state(h)) {
     e = cudaMemcpyAsync(Q, h->eng->A().hi, state_bytes(h),
                         on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream);
   } else {

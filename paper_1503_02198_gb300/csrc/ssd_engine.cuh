@@ -522,6 +522,26 @@ struct ElemGeo {
       g = tab[L::gy + k];
     }
   }
+  // the metric vector of FP i of SP line m in direction d (xi_fp or eta_fp), with
+  // the point's coordinates u = X_{i+1/2}, w = X_m at hand
+  __device__ __forceinline__ void fp_at(int d, int i, int m, T u, T w, T &vx, T &vy, T &g) const {
+    if (OTF && tab == nullptr) {
+      const T tx = (d == 0 ? e3x : e1x) + u * dx, ty = (d == 0 ? e3y : e1y) + u * dy;
+      vx = d == 0 ? ty : -ty;
+      vy = d == 0 ? -tx : tx;
+      g = T(0);
+      if (om != T(0)) {
+        const T px = x0 + u * (d == 0 ? e1x : e3x) + w * tx, py = y0 + u * (d == 0 ? e1y : e3y) + w * ty;
+        g = om * mul_sub(px, vy, py, vx);
+      }
+    } else {
+      const int k = d == 0 ? m * (N + 1) + i : i * N + m, o = d == 0 ? L::ax : L::bx;
+      const T ax = tab[o + k], ay = tab[o + L::ay - L::ax + k];
+      vx = mul_sub(c, ax, s, ay);
+      vy = mul_add(s, ax, c, ay);
+      g = tab[o + L::gx - L::ax + k];
+    }
+  }
   // Metric vectors and V_g . a at the interior FPs 1..N-1 of SP line m in
   // direction d (0: xi line at eta = X_m, 1: eta line at xi = X_m), into
   // vx/vy/vg[1..N-1].  On straight cells both directions share one form:
@@ -621,17 +641,18 @@ struct ElemGeo {
   // threads take different SPs, and constant memory serves one address at a time
   static __device__ __forceinline__ T inv_jac_at(const MeshDev &md, int f, const T *r, int sp, T xi, T eta) {
     const int ti = ((f & ~kIfaceBit) >> kZoneBits) - 1;
-    if (OTF && ti < 0) {
-      const float4 a = reinterpret_cast<const float4 *>(r)[0], b = reinterpret_cast<const float4 *>(r)[1];
-      const T xx = a.z + eta * b.z, yx = a.w + eta * b.w, xe = b.x + xi * b.z, ye = b.y + xi * b.w;
-      return recip(mul_sub(xx, ye, xe, yx));
+    if constexpr (OTF) {
+      if (ti < 0) {
+        const float4 a = reinterpret_cast<const float4 *>(r)[0], b = reinterpret_cast<const float4 *>(r)[1];
+        const T xx = a.z + eta * b.z, yx = a.w + eta * b.w, xe = b.x + xi * b.z, ye = b.y + xi * b.w;
+        return recip(mul_sub(xx, ye, xe, yx));
+      }
     }
     return ((const T *)md.geo + (size_t)ti * L::G)[L::iJ + sp];
   }
-  // gradients of xi and eta at SP (X_i, X_j): (xi_x, xi_y), (eta_x, eta_y)
-  __device__ __forceinline__ void sp_grad(int i, int j, T &xix, T &xiy, T &etx, T &ety) const {
+  // gradients of xi and eta at SP k = j N + i, at (xi, eta) = (X_i, X_j): (xi_x, xi_y), (eta_x, eta_y)
+  __device__ __forceinline__ void sp_grad_at(int k, T xi, T eta, T &xix, T &xiy, T &etx, T &ety) const {
     if (OTF && tab == nullptr) {
-      const T xi = cVB<T, N>.Xs[i], eta = cVB<T, N>.Xs[j];
       const T xx = e1x + eta * dx, yx = e1y + eta * dy, xe = e3x + xi * dx, ye = e3y + xi * dy;
       const T iJ = T(1) / mul_sub(xx, ye, xe, yx);
       xix = ye * iJ;
@@ -639,7 +660,6 @@ struct ElemGeo {
       etx = -yx * iJ;
       ety = xx * iJ;
     } else {
-      const int k = j * N + i;
       const T a = tab[L::grad + k], b = tab[L::grad + N * N + k];
       const T c2 = tab[L::grad + 2 * N * N + k], d2 = tab[L::grad + 3 * N * N + k];
       xix = mul_sub(c, a, s, b);
@@ -1012,11 +1032,42 @@ __global__ void k_fgeo(MeshDev md) {
   g[4 * N + j] = sgA * ag / SA;
 }
 
-// word of variable v at point j within an element face's 4 N values: variable
-// major, or in pairs of variables (ssd_stage.cuh)
-template <bool PAIRS, int N>
+// Order of an element face's 4 N values, and of a state's values likewise:
+// variable major; in pairs of variables (ssd_stage.cuh); or a point's four
+// variables together (ssd_viscous.cuh).
+enum { LAY_VARS = 0, LAY_PAIRS = 1, LAY_POINTS = 2 };
+// word of variable v at point j within an element face
+template <int LAY, int N>
 __device__ __forceinline__ int face_word(int v, int j) {
-  return PAIRS ? (v >> 1) * 2 * N + 2 * j + (v & 1) : v * N + j;
+  return LAY == LAY_POINTS ? 4 * j + v : LAY == LAY_PAIRS ? (v >> 1) * 2 * N + 2 * j + (v & 1) : v * N + j;
+}
+
+// four values as 16-byte accesses (p aligned to 16 bytes)
+__device__ __forceinline__ void ld4(const float *p, float *v) {
+  const float4 a = *reinterpret_cast<const float4 *>(p);
+  v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+}
+__device__ __forceinline__ void ld4(const double *p, double *v) {
+  const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
+  v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+}
+__device__ __forceinline__ void st4(float *p, const float *v) {
+  *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void st4(double *p, const double *v) {
+  reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
+  reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+}
+// a += w q for four values, in FP32 as two packed FMAs (each lane the scalar one)
+__device__ __forceinline__ void fma4(float *a, float w, const float *q) {
+  const float2 w2 = make_float2(w, w);
+  const float2 x = __ffma2_rn(w2, make_float2(q[0], q[1]), make_float2(a[0], a[1]));
+  const float2 y = __ffma2_rn(w2, make_float2(q[2], q[3]), make_float2(a[2], a[3]));
+  a[0] = x.x, a[1] = x.y, a[2] = y.x, a[3] = y.y;
+}
+__device__ __forceinline__ void fma4(double *a, double w, const double *q) {
+#pragma unroll
+  for (int v = 0; v < 4; ++v) a[v] = fma(w, q[v], a[v]);
 }
 
 // Conforming and periodic faces: one thread per face point; geometry from the
@@ -1131,7 +1182,7 @@ __device__ __forceinline__ void bface_geom(const MeshDev &md, int b, int j, T &n
 }
 
 // Boundary faces: Rusanov through the ghost state of the face's condition.
-template <typename T, int N, bool OTF, bool PAIRS = false>
+template <typename T, int N, bool OTF, int LAY = LAY_VARS>
 __device__ __forceinline__ void k_bface_point(const MeshDev &md, int t) {
   const int b = t / N, j = t - b * N;
   const int4 bf = md.bfaces[b];
@@ -1140,7 +1191,7 @@ __device__ __forceinline__ void k_bface_point(const MeshDev &md, int t) {
   const T *TR = (const T *)md.TR;
   T q[4], qg[4], qb[4];
 #pragma unroll
-  for (int v = 0; v < 4; ++v) q[v] = TR[(size_t)ef * 4 * N + face_word<PAIRS, N>(v, j)];
+  for (int v = 0; v < 4; ++v) q[v] = TR[(size_t)ef * 4 * N + face_word<LAY, N>(v, j)];
   T nx, ny, sS, vgn, ug, vg;
   bface_geom<T, N, OTF>(md, b, j, nx, ny, sS, vgn, ug, vg);
   boundary_states(md, bf.y, q, ug, vg, nx, ny, qg, qb);
@@ -1148,7 +1199,7 @@ __device__ __forceinline__ void k_bface_point(const MeshDev &md, int t) {
   rusanov(q, qg, nx, ny, vgn, pick<T>(md.gamma, md.gamma_f), Fn);
   T *CF = (T *)md.CF;
 #pragma unroll
-  for (int v = 0; v < 4; ++v) CF[(size_t)ef * 4 * N + face_word<PAIRS, N>(v, j)] = sS * Fn[v];
+  for (int v = 0; v < 4; ++v) CF[(size_t)ef * 4 * N + face_word<LAY, N>(v, j)] = sS * Fn[v];
 }
 
 // One launch for all face points of a stage: threads [0, nF N) take the
@@ -1167,7 +1218,7 @@ template <typename T, int N, bool OTF>
 __global__ void k_bfaces_pairs(MeshDev md) {
   pdl_enter();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < md.nB * N) k_bface_point<T, N, OTF, true>(md, t);
+  if (t < md.nB * N) k_bface_point<T, N, OTF, LAY_PAIRS>(md, t);
 }
 
 // Mortar coupling of Sec. 3.2.  Thread (mortar, side, p): p is a quadrature
@@ -1225,7 +1276,8 @@ struct MortShared {
 struct NoWait {
   __device__ __forceinline__ void operator()() const {}
 };
-template <typename T, int N, int MMODE, int MPB, bool PAIRS = false, class Enter = NoWait>
+template <typename T, int N, int MMODE, int MPB, int LAY = MMODE == MORTAR_RUSANOV ? LAY_VARS : LAY_POINTS,
+          class Enter = NoWait>
 __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, MortShared<T, N, MMODE, MPB> &sh,
                                                  Enter enter = Enter()) {
   constexpr int NV = MortShared<T, N, MMODE, MPB>::NV;
@@ -1254,10 +1306,8 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
       // the face's own gradient, along the radial normal (from L to R)
       const T *CQ = (const T *)md.CQ, *GT = (const T *)md.GTR;
       T q[4], g8[8], fn[4];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) q[v] = CQ[((size_t)ef * 4 + v) * N + jj];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) g8[c] = GT[((size_t)ef * 8 + c) * N + jj];
+      for (int h = 0; h < 2; ++h) ld4(GT + ((size_t)ef * N + jj) * 8 + 4 * h, g8 + 4 * h);
+      ld4(CQ + ((size_t)ef * N + jj) * 4, q);
       viscous_normal(q, g8, fcs, fsn, md, fn);
 #pragma unroll
       for (int v = 0; v < 4; ++v) sQf[lm][sd][NV - 4 + v][p] = fn[v];
@@ -1265,7 +1315,7 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
     {
       const T *TR = (const T *)md.TR;
 #pragma unroll
-      for (int v = 0; v < 4; ++v) sQf[lm][sd][v][p] = TR[(size_t)ef * 4 * N + face_word<PAIRS, N>(v, jj)];
+      for (int v = 0; v < 4; ++v) sQf[lm][sd][v][p] = TR[(size_t)ef * 4 * N + face_word<LAY, N>(v, jj)];
     }
   };
   for (int k = threadIdx.x; k < N * N; k += blockDim.x) {
@@ -1398,11 +1448,11 @@ __device__ __forceinline__ void mortar_flux_body(const MeshDev &md, int blk, Mor
   }
 }
 
-template <typename T, int N, int MMODE, bool PAIRS = false>
+template <typename T, int N, int MMODE, int LAY>
 __global__ void __launch_bounds__(MortCfg<N>::THREADS) k_mortar_flux(MeshDev md) {
   pdl_enter();
   __shared__ MortShared<T, N, MMODE, MortCfg<N>::MPB> sh;
-  mortar_flux_body<T, N, MMODE, MortCfg<N>::MPB, PAIRS>(md, blockIdx.x, sh);
+  mortar_flux_body<T, N, MMODE, MortCfg<N>::MPB, LAY>(md, blockIdx.x, sh);
 }
 
 // Sum of the mortar contributions of each interface face (fixed order: the
@@ -1457,7 +1507,7 @@ __device__ __forceinline__ bool gather_sum(const MeshDev &md, int fq, int p, T *
 // values [face][variable][point], element stride `stride`) in the tile's
 // shared copy; with `global` also in CQ / CF.  Returns whether the tile had
 // an interface cell (then the caller synchronises before reading the tile).
-template <typename T, int N, int GMODE>
+template <typename T, int N, int GMODE, int LAY = LAY_VARS>
 __device__ __forceinline__ bool gather_tile(const MeshDev &md, int e0, int ne, const int *sEF, T *tile, int stride,
                                             bool global, int nthreads) {
   // the tile's flags in 16-byte groups (a tile's flags are copied in whole
@@ -1479,11 +1529,11 @@ __device__ __forceinline__ bool gather_tile(const MeshDev &md, int e0, int ne, c
     int ef, j;
     if (!gather_sum<T, N, GMODE>(md, fq, rev ? N - 1 - jj : jj, val, ef, j)) continue;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) tile[le * stride + (f * 4 + v) * N + jj] = val[v];
+    for (int v = 0; v < 4; ++v) tile[le * stride + f * 4 * N + face_word<LAY, N>(v, jj)] = val[v];
     if (global) {
       T *dst = (T *)(GMODE == GATHER_Q ? md.CQ : md.CF);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) dst[((size_t)ef * 4 + v) * N + j] = val[v];
+      for (int v = 0; v < 4; ++v) dst[(size_t)ef * 4 * N + face_word<LAY, N>(v, j)] = val[v];
     }
   }
   return true;
@@ -2416,6 +2466,11 @@ struct EngineImpl : Engine {
         return;
       }
     }
+    if (md.viscous) {
+      const int n = (int)(nval / 4);
+      k_split_points<T, N * N><<<(n + 511) / 512, 256, 0, s>>>(Q, (T *)sA[0], (T *)sA[1], n);
+      return;
+    }
     if (DF)
       k_split<<<(unsigned)((nval + 255) / 256), 256, 0, s>>>(Q, (float *)sA[0], (float *)sA[1], nval);
     else if (OTF)
@@ -2430,6 +2485,11 @@ struct EngineImpl : Engine {
         k_join_pairs<N * N><<<(n + 1023) / 1024, 256, 0, s>>>((const float2 *)sA[0], (const float2 *)sA[1], Q, n);
         return;
       }
+    }
+    if (md.viscous) {
+      const int n = (int)(nval / 4);
+      k_join_points<T, N * N><<<(n + 511) / 512, 256, 0, s>>>((const T *)sA[0], (const T *)sA[1], Q, n);
+      return;
     }
     if (OTF)
       k_join<<<(unsigned)((nval + 255) / 256), 256, 0, s>>>((const float *)sA[0], (const float *)sA[1], Q, nval);
@@ -2549,6 +2609,10 @@ struct EngineImpl : Engine {
         return;
       }
     }
+    if (md.viscous) {
+      launch_pdl(k_trace_points<T, N>, (md.E * 4 * N + 255) / 256, 256, 0, s, md, (const T *)q.hi);
+      return;
+    }
     const int n = md.E * 16 * N;
     launch_pdl(k_trace<T, N>, (n + 255) / 256, 256, 0, s, md, (const T *)q.hi);
   }
@@ -2575,10 +2639,10 @@ struct EngineImpl : Engine {
   // the mortar flux as its own launch; the gather of its contributions into
   // each interface face is done by the kernel that reads the result
   // (gather_tile in k_volume, k_volume_visc, k_grad_trace)
-  template <int MMODE, bool PAIRS = false>
+  template <int MMODE, int LAY = MMODE == MORTAR_RUSANOV ? LAY_VARS : LAY_POINTS>
   void mortar_flux(const MeshDev &md, cudaStream_t s) {
     constexpr int MPB = MortCfg<N>::MPB;
-    launch_pdl(k_mortar_flux<T, N, MMODE, PAIRS>, (md.nM + MPB - 1) / MPB, MortCfg<N>::THREADS, 0, s, md);
+    launch_pdl(k_mortar_flux<T, N, MMODE, LAY>, (md.nM + MPB - 1) / MPB, MortCfg<N>::THREADS, 0, s, md);
   }
 
   // a face pass fused with the mortar flux of the same pass (meshes with an
@@ -2640,7 +2704,7 @@ struct EngineImpl : Engine {
   void mortars(const MeshDev &md, cudaStream_t s) override {
     if (md.nL > 0 && !fuse_faces_mortar) {
       if (md.viscous) mortar_flux<MORTAR_RUSANOV_FV>(md, s);
-      else if (md.frec) mortar_flux<MORTAR_RUSANOV, true>(md, s);
+      else if (md.frec) mortar_flux<MORTAR_RUSANOV, LAY_PAIRS>(md, s);
       else mortar_flux<MORTAR_RUSANOV>(md, s);
     }
   }

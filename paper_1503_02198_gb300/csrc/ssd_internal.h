@@ -141,8 +141,9 @@ struct MeshDev {
   // and its tiles in working order; null where it does not run
   const float4 *frec, *fgp;
   const int *tord;
-  void *CQ, *GTR;         // viscous: T [E][4][4][N] common solution, [E][4][8][N] gradient traces
-  void *GSP;              // viscous: T [E][8][N][N] gradients at the SPs (x then y, 4 variables each)
+  // (viscous meshes: a point's values together, see ssd_viscous.cuh)
+  void *CQ, *GTR;         // viscous: T [E][4][N][4] common solution, [E][4][N][8] gradient traces
+  void *GSP;              // viscous: T [E][2][N*N][4] gradients at the SPs (x then y, 4 variables each)
   void *fgeo;             // T [nF][5][N] conforming-face geometry at t = 0: unit normal
                           // (x, y) out of side A, sigma_A |S_A|, sigma_B |S_B|, V_g . n
   DevClock *clk;

@@ -337,11 +337,11 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
   };
   auto couple = [&](int c) {
     if (c < nmort) {
-      mortar_flux_body<float, N, MORTAR_RUSANOV, EPB, true>(md, c, *(typename C::Mort *)(smem + C::O_QLO), enter);
+      mortar_flux_body<float, N, MORTAR_RUSANOV, EPB, LAY_PAIRS>(md, c, *(typename C::Mort *)(smem + C::O_QLO), enter);
     } else {
       enter();
       const int t = (c - nmort) * NT + threadIdx.x;
-      if (t < md.nB * N) k_bface_point<float, N, true, true>(md, t);
+      if (t < md.nB * N) k_bface_point<float, N, true, LAY_PAIRS>(md, t);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
     } else {
       const float *cf = (const float *)md.CF + (size_t)ef * 4 * N;
 #pragma unroll
-      for (int v = 0; v < 4; ++v) val[v] = cf[face_word<true, N>(v, mline)];
+      for (int v = 0; v < 4; ++v) val[v] = cf[face_word<LAY_PAIRS, N>(v, mline)];
     }
   };
 

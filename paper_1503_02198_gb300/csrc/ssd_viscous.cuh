@@ -25,6 +25,18 @@
 //                              the stored SP gradients), divergence, Runge-Kutta
 //                              update, traces; persistent, tiles fed by 1-D
 //                              bulk copies one tile ahead
+//
+// Layout.  On this path the values of a point lie together: the state is
+// [E][N^2][4], traces, common solution and common fluxes [E][4 faces][N][4], SP
+// gradients [E][2][N^2][4] and gradient traces [E][4][N][8] (x then y).  A point's
+// state is one 16-byte access (two in FP64) and two packed FP32x2 operands, where
+// one variable at a time took four loads and four FMAs; the kernels here were
+// bound by instructions and latency with their tiles in L2, not by bytes.  The
+// state crosses the ABI as [E][4][N][N] and is converted with the double-float
+// split.  us a step, one variable at a time ->
+// points (FP32): 14,752 cells N = 4, five stages 192 -> 152; 20,096 cells N = 5
+// 181 -> 164 (the volume kernel's warp instructions 18.2 -> 12.3 million, now
+// barrier and shared-load latency with 20 warps per SM).
 #pragma once
 
 namespace ssd {
@@ -62,6 +74,63 @@ __device__ __forceinline__ void viscous_flux(const T *q, const T *qx, const T *q
   G[3] = -fma(u, txy, mul_add(v, tyy, kr, Ty));
 }
 
+// ---- state conversion and traces ----------------------------------------------
+
+// FP64 state [E][4][N^2] -> the points layout (a double-float pair, a float or a
+// double per value); thread = one SP
+template <typename T, int NN>
+__global__ void k_split_points(const double *__restrict__ Q, T *hi, T *lo, int n) {
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int t = (blockIdx.x * 2 + u) * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    const size_t g = (size_t)(t / NN) * 4 * NN + t % NN;
+    T h[4], l[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const double x = Q[g + v * NN];
+      h[v] = (T)x;
+      l[v] = (T)(x - (double)h[v]);
+    }
+    st4(hi + (size_t)t * 4, h);
+    if (lo) st4(lo + (size_t)t * 4, l);
+  }
+}
+
+template <typename T, int NN>
+__global__ void k_join_points(const T *__restrict__ hi, const T *__restrict__ lo, double *Q, int n) {
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int t = (blockIdx.x * 2 + u) * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    const size_t g = (size_t)(t / NN) * 4 * NN + t % NN;
+    T h[4], l[4] = {0, 0, 0, 0};
+    ld4(hi + (size_t)t * 4, h);
+    if (lo) ld4(lo + (size_t)t * 4, l);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) Q[g + v * NN] = lo ? (double)h[v] + (double)l[v] : (double)h[v];
+  }
+}
+
+// face traces of a state; thread = one face point
+template <typename T, int N>
+__global__ void k_trace_points(MeshDev md, const T *__restrict__ Q) {
+  pdl_enter();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= md.E * 4 * N) return;
+  const int e = t / (4 * N), r = t - e * 4 * N, f = r / N, j = r - f * N;
+  const VolBasis<T, N> &B = cVB<T, N>;
+  const T *q = Q + (size_t)e * 4 * N * N;
+  T acc[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    T v[4];
+    ld4(q + 4 * ((f == 0 || f == 2) ? k * N + j : j * N + k), v);
+    fma4(acc, (f == 1 || f == 2) ? B.H1[k] : B.H0[k], v);
+  }
+  st4((T *)md.TR + (size_t)t * 4, acc);
+}
+
 // ---- common solution -------------------------------------------------------
 
 template <typename T, int N>
@@ -71,12 +140,13 @@ __device__ __forceinline__ void k_face_cq_point(const MeshDev &md, int t) {
   const int efA = fc.x, efB = fc.y, jB = fc.z ? N - 1 - j : j;
   const T *TR = (const T *)md.TR;
   T *CQ = (T *)md.CQ;
+  T a[4], b[4], c[4];
+  ld4(TR + ((size_t)efA * N + j) * 4, a);
+  ld4(TR + ((size_t)efB * N + jB) * 4, b);
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const T c = T(0.5) * (TR[((size_t)efA * 4 + v) * N + j] + TR[((size_t)efB * 4 + v) * N + jB]);
-    CQ[((size_t)efA * 4 + v) * N + j] = c;
-    CQ[((size_t)efB * 4 + v) * N + jB] = c;
-  }
+  for (int v = 0; v < 4; ++v) c[v] = T(0.5) * (a[v] + b[v]);
+  st4(CQ + ((size_t)efA * N + j) * 4, c);
+  st4(CQ + ((size_t)efB * N + jB) * 4, c);
 }
 
 // boundary faces: the common solution is the state on the boundary
@@ -87,13 +157,11 @@ __device__ __forceinline__ void k_bface_cq_point(const MeshDev &md, int t) {
   const int ef = bf.x;
   const T *TR = (const T *)md.TR;
   T q[4], qg[4], qb[4];
-#pragma unroll
-  for (int v = 0; v < 4; ++v) q[v] = TR[((size_t)ef * 4 + v) * N + j];
+  ld4(TR + ((size_t)ef * N + j) * 4, q);
   T nx, ny, sS, vgn, ug, vg;
   bface_geom<T, N, OTF>(md, b, j, nx, ny, sS, vgn, ug, vg);
   boundary_states(md, bf.y, q, ug, vg, nx, ny, qg, qb);
-#pragma unroll
-  for (int v = 0; v < 4; ++v) ((T *)md.CQ)[((size_t)ef * 4 + v) * N + j] = qb[v];
+  st4((T *)md.CQ + ((size_t)ef * N + j) * 4, qb);
 }
 
 // common solution at all face points of a stage (conforming, then boundary)
@@ -119,41 +187,38 @@ struct VisCfg {
 };
 
 // Gradients at the SPs of a tile (thread per SP line, then per SP): on
-// return sDx / sDe hold Q_x / Q_y, and gsp (the tile's rows of GSP,
-// [element][8][N^2]) the same.  The caller synchronises before and after.
+// return sDx / sDe hold Q_x / Q_y [element][SP][4], and gsp (the tile's rows of
+// GSP, [element][2][SP][4]) the same.  The caller synchronises before and after.
 template <typename T, int N, bool OTF>
-__device__ __forceinline__ void tile_gradients(const MeshDev &md, int e0, int ne, T (*sQ)[4][N * N],
-                                               T (*sCQ)[16 * N], T (*sDx)[4][N * N], T (*sDe)[4][N * N],
-                                               const T *zt, const int *sEF, const T *sEG, T *gsp) {
+__device__ __forceinline__ void tile_gradients(const MeshDev &md, int e0, int ne, const T *sQ, const T *sCQ, T *sDx,
+                                               T *sDe, const T *zt, const int *sEF, const T *sEG, const T *sXs,
+                                               T *gsp) {
   constexpr int NN = N * N, NT = VisCfg<T, N>::THREADS;
   const VolBasis<T, N> &B = cVB<T, N>;
   const int le = threadIdx.x / (2 * N);
   const int r = threadIdx.x - le * 2 * N;
   const int d = r / N, m = r - d * N;
   if (le < ne) {
+    // the line's N + 1 flux-point values, the common solution at its ends
+    T val[N + 1][4], qv[N][4];
+    ld4(sCQ + (le * 4 + (d == 0 ? 3 : 0)) * 4 * N + 4 * m, val[0]);
+    ld4(sCQ + (le * 4 + (d == 0 ? 1 : 2)) * 4 * N + 4 * m, val[N]);
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      T val[N + 1], qv[N];
-      val[0] = sCQ[le][((d == 0 ? 3 : 0) * 4 + v) * N + m];
-      val[N] = sCQ[le][((d == 0 ? 1 : 2) * 4 + v) * N + m];
-      // the line's N values, read once for all its flux points
+    for (int k = 0; k < N; ++k) ld4(sQ + 4 * (le * NN + (d == 0 ? m * N + k : k * N + m)), qv[k]);
 #pragma unroll
-      for (int k = 0; k < N; ++k) qv[k] = sQ[le][v][d == 0 ? m * N + k : k * N + m];
+    for (int i = 1; i < N; ++i) {
 #pragma unroll
-      for (int i = 1; i < N; ++i) {
-        T acc = 0;
+      for (int v = 0; v < 4; ++v) val[i][v] = 0;
 #pragma unroll
-        for (int k = 0; k < N; ++k) acc += qv[k] * B.Hf[i * N + k];
-        val[i] = acc;
-      }
+      for (int k = 0; k < N; ++k) fma4(val[i], B.Hf[i * N + k], qv[k]);
+    }
+    T *o = d == 0 ? sDx : sDe;  // d/dxi at SP (k, m), or d/deta at SP (m, k)
 #pragma unroll
-      for (int k = 0; k < N; ++k) {
-        T acc = 0;
+    for (int k = 0; k < N; ++k) {
+      T acc[4] = {0, 0, 0, 0};
 #pragma unroll
-        for (int i = 0; i <= N; ++i) acc += B.Dm[k * (N + 1) + i] * val[i];
-        if (d == 0) sDx[le][v][m * N + k] = acc;   // d/dxi at SP (k, m)
-        else sDe[le][v][k * N + m] = acc;          // d/deta at SP (m, k)
-      }
+      for (int i = 0; i <= N; ++i) fma4(acc, B.Dm[k * (N + 1) + i], val[i]);
+      st4(o + 4 * (le * NN + (d == 0 ? m * N + k : k * N + m)), acc);
     }
   }
   __syncthreads();
@@ -161,18 +226,19 @@ __device__ __forceinline__ void tile_gradients(const MeshDev &md, int e0, int ne
     const int l2 = idx / NN, sp = idx - l2 * NN;
     ElemGeo<T, N, OTF> G;
     G.load_rec(md, e0 + l2, sEF[l2], sEG + l2 * 8, zt);
-    T xix, xiy, etx, ety;
-    G.sp_grad(sp % N, sp / N, xix, xiy, etx, ety);
-    T *g = gsp + (size_t)l2 * 8 * NN + sp;
+    T xix, xiy, etx, ety, a[4], b[4], gx[4], gy[4];
+    G.sp_grad_at(sp, sXs[sp % N], sXs[sp / N], xix, xiy, etx, ety);
+    ld4(sDx + 4 * idx, a);
+    ld4(sDe + 4 * idx, b);
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      const T a = sDx[l2][v][sp], b = sDe[l2][v][sp];
-      const T gx = mul_add(xix, a, etx, b), gy = mul_add(xiy, a, ety, b);
-      sDx[l2][v][sp] = gx;
-      sDe[l2][v][sp] = gy;
-      g[v * NN] = gx;
-      g[(4 + v) * NN] = gy;
+      gx[v] = mul_add(xix, a[v], etx, b[v]);
+      gy[v] = mul_add(xiy, a[v], ety, b[v]);
     }
+    st4(sDx + 4 * idx, gx);
+    st4(sDe + 4 * idx, gy);
+    st4(gsp + (size_t)(l2 * 2 * NN + sp) * 4, gx);
+    st4(gsp + (size_t)(l2 * 2 * NN + NN + sp) * 4, gy);
   }
 }
 
@@ -188,12 +254,13 @@ struct GradCfg {
   static constexpr int STAGE = ((O_EF + EPB * 4) + 127) / 128 * 128;
   static constexpr int O_DX = 2 * STAGE, O_DE = O_DX + EPB * QE;
   static constexpr int O_BAR = ((O_DE + EPB * QE) + 15) / 16 * 16;
-  static constexpr int SMEM = O_BAR + 2 * 8;
+  static constexpr int O_XS = O_BAR + 2 * 8;  // the solution points
+  static constexpr int SMEM = O_XS + N * (int)sizeof(T);
   static_assert(QE % 16 == 0 && CE % 16 == 0, "bulk-copy sizes and alignment");
   static_assert(SMEM <= 227 * 1024, "dynamic shared memory of one CTA");
 };
 
-// SP gradients GSP [E][8][N][N] and gradient traces GTR [E][4 faces][8][N]
+// SP gradients GSP [E][2][N^2][4] and gradient traces GTR [E][4 faces][N][8]
 // (component v = dQ_v/dx, 4 + v = dQ_v/dy).  Persistent: each CTA walks
 // tiles; thread 0 issues the next tile's state and common solution (two 1-D
 // bulk copies) into the other stage while the CTA computes the current one.
@@ -204,8 +271,7 @@ __global__ void __launch_bounds__(GradCfg<T, N>::THREADS) k_grad_trace(Src src, 
   constexpr int EPB = C::EPB, NT = C::THREADS, NN = N * N;
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t *bar = (uint64_t *)(smem + C::O_BAR);
-  T(*sDx)[4][NN] = (T(*)[4][NN])(smem + C::O_DX);
-  T(*sDe)[4][NN] = (T(*)[4][NN])(smem + C::O_DE);
+  T *sDx = (T *)(smem + C::O_DX), *sDe = (T *)(smem + C::O_DE), *sXs = (T *)(smem + C::O_XS);
   // the state of the stage (the item's case's input state), the common
   // solution, the cell records (on-the-fly path) and flags; the flags are
   // copied in whole groups of 4 (16 bytes), within the tile-padded array
@@ -236,6 +302,7 @@ __global__ void __launch_bounds__(GradCfg<T, N>::THREADS) k_grad_trace(Src src, 
   int item = blockIdx.x;
   if (threadIdx.x == 0 && item < nitems) issue(item, 0);
   const VolBasis<T, N> &B = cVB<T, N>;
+  if (threadIdx.x < N) sXs[threadIdx.x] = B.Xs[threadIdx.x];  // (read after the first barrier below)
   const int le = threadIdx.x / (2 * N);
   const int r = threadIdx.x - le * 2 * N;
   const int d = r / N, m = r - d * N;
@@ -259,34 +326,32 @@ __global__ void __launch_bounds__(GradCfg<T, N>::THREADS) k_grad_trace(Src src, 
       return;
     }
     unsigned char *sb = smem + st * C::STAGE;
-    T(*sQ)[4][NN] = (T(*)[4][NN])(sb + C::O_Q);
-    T(*sCQ)[16 * N] = (T(*)[16 * N])(sb + C::O_C);
+    const T *sQ = (const T *)(sb + C::O_Q), *sCQ = (const T *)(sb + C::O_C);
     const T *sEG = (const T *)(sb + C::O_EG);
     const int *sEF = (const int *)(sb + C::O_EF);
     const int e0 = tile * EPB;
     const int ne = min(EPB, md.E - e0);
     // the tile's interface faces: their common solution from the mortar
     // contributions, also into CQ for the viscous mortar pass that follows
-    if (gather_tile<T, N, GATHER_Q>(md, e0, ne, sEF, (T *)(sb + C::O_C), 16 * N, true, NT)) __syncthreads();
+    if (gather_tile<T, N, GATHER_Q, LAY_POINTS>(md, e0, ne, sEF, (T *)(sb + C::O_C), 16 * N, true, NT)) __syncthreads();
     // the SP gradients, also stored for the volume kernel of this stage
-    tile_gradients<T, N, OTF>(md, e0, ne, sQ, sCQ, sDx, sDe, zt, sEF, sEG, (T *)md.GSP + (size_t)e0 * 8 * NN);
+    tile_gradients<T, N, OTF>(md, e0, ne, sQ, sCQ, sDx, sDe, zt, sEF, sEG, sXs, (T *)md.GSP + (size_t)e0 * 8 * NN);
     __syncthreads();
     if (le < ne) {
-      T *g = (T *)md.GTR + (size_t)(e0 + le) * 32 * N;
+      T *g = (T *)md.GTR + (size_t)(e0 + le) * 32 * N + 8 * m;
       const int fa = d == 0 ? 3 : 0, fb = d == 0 ? 1 : 2;
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const int v = c & 3;
-        T a0 = 0, a1 = 0;
+      for (int c = 0; c < 2; ++c) {
+        T a0[4] = {0, 0, 0, 0}, a1[4] = {0, 0, 0, 0};
 #pragma unroll
         for (int k = 0; k < N; ++k) {
-          const int sp = d == 0 ? m * N + k : k * N + m;
-          const T val = c < 4 ? sDx[le][v][sp] : sDe[le][v][sp];
-          a0 += val * B.H0[k];
-          a1 += val * B.H1[k];
+          T val[4];
+          ld4((c ? sDe : sDx) + 4 * (le * NN + (d == 0 ? m * N + k : k * N + m)), val);
+          fma4(a0, B.H0[k], val);
+          fma4(a1, B.H1[k], val);
         }
-        g[(fa * 8 + c) * N + m] = a0;
-        g[(fb * 8 + c) * N + m] = a1;
+        st4(g + fa * 8 * N + 4 * c, a0);
+        st4(g + fb * 8 * N + 4 * c, a1);
       }
     }
     // every read of this tile's stage and of the gradient arrays is done
@@ -314,16 +379,14 @@ __device__ __forceinline__ void k_face_visc_point(const MeshDev &md, int t) {
   const int efA = fc.x, efB = fc.y, jB = fc.z ? N - 1 - j : j;
   const T *TR = (const T *)md.TR, *CQ = (const T *)md.CQ, *GT = (const T *)md.GTR;
   T qA[4], qB[4], qc[4], gA[8], gB[8];
+  const size_t pA = (size_t)efA * N + j, pB = (size_t)efB * N + jB;
+  ld4(TR + pA * 4, qA);
+  ld4(TR + pB * 4, qB);
+  ld4(CQ + pA * 4, qc);
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    qA[v] = TR[((size_t)efA * 4 + v) * N + j];
-    qB[v] = TR[((size_t)efB * 4 + v) * N + jB];
-    qc[v] = CQ[((size_t)efA * 4 + v) * N + j];
-  }
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    gA[c] = GT[((size_t)efA * 8 + c) * N + j];
-    gB[c] = GT[((size_t)efB * 8 + c) * N + jB];
+  for (int h = 0; h < 2; ++h) {
+    ld4(GT + pA * 8 + 4 * h, gA + 4 * h);
+    ld4(GT + pB * 8 + 4 * h, gB + 4 * h);
   }
   const T *g = (const T *)md.fgeo + (size_t)fi * 5 * N;
   T nx = g[j], ny = g[N + j];
@@ -341,12 +404,15 @@ __device__ __forceinline__ void k_face_visc_point(const MeshDev &md, int t) {
   viscous_normal(qc, gA, nx, ny, md, va);
   viscous_normal(qc, gB, nx, ny, md, vb);
   T *CF = (T *)md.CF;
+  T fA[4], fB[4];
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     const T f = Fn[v] + T(0.5) * (va[v] + vb[v]);
-    CF[((size_t)efA * 4 + v) * N + j] = sA * f;
-    CF[((size_t)efB * 4 + v) * N + jB] = -sB * f;
+    fA[v] = sA * f;
+    fB[v] = -sB * f;
   }
+  st4(CF + pA * 4, fA);
+  st4(CF + pB * 4, fB);
 }
 
 // boundary faces: Rusanov through the ghost state plus the viscous flux of the
@@ -358,10 +424,9 @@ __device__ __forceinline__ void k_bface_visc_point(const MeshDev &md, int t) {
   const int ef = bf.x;
   const T *TR = (const T *)md.TR, *GT = (const T *)md.GTR;
   T q[4], qg[4], qb[4], g8[8];
+  ld4(TR + ((size_t)ef * N + j) * 4, q);
 #pragma unroll
-  for (int v = 0; v < 4; ++v) q[v] = TR[((size_t)ef * 4 + v) * N + j];
-#pragma unroll
-  for (int c = 0; c < 8; ++c) g8[c] = GT[((size_t)ef * 8 + c) * N + j];
+  for (int h = 0; h < 2; ++h) ld4(GT + ((size_t)ef * N + j) * 8 + 4 * h, g8 + 4 * h);
   T nx, ny, sS, vgn, ug, vg;
   bface_geom<T, N, OTF>(md, b, j, nx, ny, sS, vgn, ug, vg);
   boundary_states(md, bf.y, q, ug, vg, nx, ny, qg, qb);
@@ -370,7 +435,8 @@ __device__ __forceinline__ void k_bface_visc_point(const MeshDev &md, int t) {
   viscous_normal(qb, g8, nx, ny, md, fv, bf.y != SD_BC_ADIABATIC);
   T *CF = (T *)md.CF;
 #pragma unroll
-  for (int v = 0; v < 4; ++v) CF[((size_t)ef * 4 + v) * N + j] = sS * (Fn[v] + fv[v]);
+  for (int v = 0; v < 4; ++v) Fn[v] = sS * (Fn[v] + fv[v]);
+  st4(CF + ((size_t)ef * N + j) * 4, Fn);
 }
 
 // common inviscid + viscous fluxes at all face points of a stage
@@ -401,18 +467,23 @@ struct VisVolCfg {
   static constexpr int O_EF = O_EG + EPB * GEE;
   static constexpr int STAGE = ((O_EF + EPB * 4) + 127) / 128 * 128;
   // fluxes [EPB][2 directions][N lines][LS]: a line's N - 1 interior points,
-  // 4 values each; the odd line stride puts neighbouring lines in different banks
-  static constexpr int LS = 4 * (N - 1) + 1;
+  // 4 values each; a stride of an odd number of points puts eight neighbouring
+  // lines in different banks
+  static constexpr int LS = 4 * ((N - 1) | 1);
   static constexpr int O_FL = 2 * STAGE;
-  static constexpr int O_W = O_FL + (EPB * 2 * N * LS * (int)sizeof(T) + 15) / 16 * 16;  // Hf, then Dm
-  static constexpr int O_BAR = (O_W + 2 * N * (N + 1) * (int)sizeof(T) + 15) / 16 * 16;
+  static constexpr int O_W = O_FL + (EPB * 2 * N * LS * (int)sizeof(T) + 15) / 16 * 16;  // Hf, Dm, Xs, Xf
+  static constexpr int O_BAR = (O_W + (2 * N * (N + 1) + 2 * N + 1) * (int)sizeof(T) + 15) / 16 * 16;
   static constexpr int SMEM = O_BAR + 2 * 8;
   static_assert(QE % 16 == 0 && GE % 16 == 0 && CE % 16 == 0, "bulk-copy sizes and alignment");
   static_assert(SMEM <= 227 * 1024 && THREADS <= 1024, "one CTA");
-  // resident CTAs per SM the register budget is set for: about 24 warps, or
-  // what the shared memory admits
+  // resident CTAs per SM the register budget is set for (warps per SM), or what
+  // the shared memory admits.  us a step for 16 / 20 / 25 / 32 warps: FP32 N = 3
+  // (288 cells) 55.7 / 55.8 / 56.4 / 60.0, N = 4 (14,752 cells, five stages)
+  // 176 / 168 / 160 / 161, N = 5 (20,096 cells) 179 / 168 / 173 / 176; FP64 N = 5
+  // 1856 / 1865 / 1865 / 1866
   static constexpr int WARPS = (THREADS + 31) / 32;
-  static constexpr int BY_WARPS = 32 / WARPS > 0 ? 32 / WARPS : 1;
+  static constexpr int BUDGET = sizeof(T) == 4 ? (N == 4 ? 25 : 20) : 16;
+  static constexpr int BY_WARPS = BUDGET / WARPS > 0 ? BUDGET / WARPS : 1;
   static constexpr int BY_SMEM = 228 * 1024 / (SMEM + 1024);
   static constexpr int MINB = BY_WARPS < BY_SMEM ? BY_WARPS : (BY_SMEM > 0 ? BY_SMEM : 1);
 };
@@ -432,7 +503,7 @@ __global__ void __launch_bounds__(VisVolCfg<T, N>::THREADS, VisVolCfg<T, N>::MIN
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t *bar = (uint64_t *)(smem + C::O_BAR);
   T *sFl = (T *)(smem + C::O_FL);
-  T *sHf = (T *)(smem + C::O_W), *sDm = sHf + (N + 1) * N;
+  T *sHf = (T *)(smem + C::O_W), *sDm = sHf + (N + 1) * N, *sXs = sDm + (N + 1) * N, *sXf = sXs + N;
   const VolBasis<T, N> &B = cVB<T, N>;
   // the state, the SP gradients that k_grad_trace formed from it in this
   // stage, and the common fluxes of tile tl into stage st
@@ -465,6 +536,8 @@ __global__ void __launch_bounds__(VisVolCfg<T, N>::THREADS, VisVolCfg<T, N>::MIN
   for (int k = threadIdx.x; k < (N + 1) * N; k += NT) {
     sHf[k] = B.Hf[k];
     sDm[k] = B.Dm[k];
+    if (k < N) sXs[k] = B.Xs[k];
+    if (k <= N) sXf[k] = B.Xf[k];
   }
   __syncthreads();
   int item = blockIdx.x;
@@ -508,15 +581,14 @@ __global__ void __launch_bounds__(VisVolCfg<T, N>::THREADS, VisVolCfg<T, N>::MIN
       return;
     }
     unsigned char *sb = smem + st * C::STAGE;
-    T(*sQ)[4][NN] = (T(*)[4][NN])(sb + C::O_Q);
-    const T(*sG)[8][NN] = (const T(*)[8][NN])(sb + C::O_G);
-    const T(*sCF)[16 * N] = (const T(*)[16 * N])(sb + C::O_C);
+    T *sQ = (T *)(sb + C::O_Q);                                                     // [EPB][NN][4]
+    const T *sG = (const T *)(sb + C::O_G), *sCF = (const T *)(sb + C::O_C);        // [EPB][2][NN][4], [EPB][4][N][4]
     const T *sEG = (const T *)(sb + C::O_EG);
     const int *sEF = (const int *)(sb + C::O_EF);
     const int e0 = tile * EPB;
     const int ne = min(EPB, md.E - e0);
     // the tile's interface faces: their common fluxes from the mortar contributions
-    if (gather_tile<T, N, GATHER_FLUX>(md, e0, ne, sEF, (T *)(sb + C::O_C), 16 * N, false, NT)) __syncthreads();
+    if (gather_tile<T, N, GATHER_FLUX, LAY_POINTS>(md, e0, ne, sEF, (T *)(sb + C::O_C), 16 * N, false, NT)) __syncthreads();
     // ---- phase 1: one thread per interior flux point: Q and its gradients
     // interpolated to the point (Eq. Qt), the inviscid ALE flux and the
     // viscous flux (Sec. 2.1) transformed with the point's metric vector,
@@ -525,31 +597,28 @@ __global__ void __launch_bounds__(VisVolCfg<T, N>::THREADS, VisVolCfg<T, N>::MIN
       ElemGeo<T, N, OTF> G;
       G.load_rec(md, e0 + le, sEF[le], sEG + le * 8, zt);
       const T *h = sHf + fi * N;
-      T qf[4], g8[8];
+      T qf[4] = {0, 0, 0, 0}, g8[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        T a = 0, bx = 0, by = 0;
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-          const int sp = d == 0 ? m * N + k : k * N + m;
-          a = fma(sQ[le][v][sp], h[k], a);
-          bx = fma(sG[le][v][sp], h[k], bx);
-          by = fma(sG[le][4 + v][sp], h[k], by);
-        }
-        qf[v] = a;
-        g8[v] = bx;
-        g8[4 + v] = by;
+      for (int k = 0; k < N; ++k) {
+        const int sp = d == 0 ? m * N + k : k * N + m;
+        T q[4], gx[4], gy[4];
+        ld4(sQ + 4 * (le * NN + sp), q);
+        ld4(sG + 4 * (le * 2 * NN + sp), gx);
+        ld4(sG + 4 * (le * 2 * NN + NN + sp), gy);
+        fma4(qf, h[k], q);
+        fma4(g8, h[k], gx);
+        fma4(g8 + 4, h[k], gy);
       }
       T vx, vy, vg;
-      if (d == 0) G.xi_fp(fi, m, vx, vy, vg);
-      else G.eta_fp(m, fi, vx, vy, vg);
+      G.fp_at(d, fi, m, sXf[fi], sXs[m], vx, vy, vg);
       const T p = pressure_of(qf, gm1);
       T f[4], Fv[4], Gv[4];
       normal_flux(qf, p, vx, vy, vg, f);
       viscous_flux(qf, g8, g8 + 4, md, Fv, Gv);
       T *o = sFl + ((le * 2 + d) * N + m) * C::LS + (fi - 1) * 4;
 #pragma unroll
-      for (int v = 0; v < 4; ++v) o[v] = fma(vx, Fv[v], fma(vy, Gv[v], f[v]));
+      for (int v = 0; v < 4; ++v) f[v] = fma(vx, Fv[v], fma(vy, Gv[v], f[v]));
+      st4(o, f);
     }
     __syncthreads();
     // (RF + RG)[v] at SP sp = (i, j) of element l2: each direction's
@@ -559,167 +628,110 @@ __global__ void __launch_bounds__(VisVolCfg<T, N>::THREADS, VisVolCfg<T, N>::MIN
       const int i = sp % N, j = sp / N;
       const T *fx = sFl + ((l2 * 2 + 0) * N + j) * C::LS, *fe = sFl + ((l2 * 2 + 1) * N + i) * C::LS;
       const T *wx = sDm + i * (N + 1), *we = sDm + j * (N + 1);
+      const T *cf = sCF + l2 * 16 * N;
+      T a[4] = {0, 0, 0, 0}, b[4] = {0, 0, 0, 0}, t[4];
+      ld4(cf + (3 * N + j) * 4, t);
+      fma4(a, wx[0], t);
+      ld4(cf + (0 * N + i) * 4, t);
+      fma4(b, we[0], t);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        T a = mul_rn(wx[0], sCF[l2][(3 * 4 + v) * N + j]);
-        T b = mul_rn(we[0], sCF[l2][(0 * 4 + v) * N + i]);
+      for (int l = 1; l < N; ++l) {
+        ld4(fx + (l - 1) * 4, t);
+        fma4(a, wx[l], t);
+        ld4(fe + (l - 1) * 4, t);
+        fma4(b, we[l], t);
+      }
+      ld4(cf + (1 * N + j) * 4, t);
+      fma4(a, wx[N], t);
+      ld4(cf + (2 * N + i) * 4, t);
+      fma4(b, we[N], t);
 #pragma unroll
-        for (int l = 1; l < N; ++l) {
-          a = fma(wx[l], fx[(l - 1) * 4 + v], a);
-          b = fma(we[l], fe[(l - 1) * 4 + v], b);
-        }
-        a = fma(wx[N], sCF[l2][(1 * 4 + v) * N + j], a);
-        b = fma(we[N], sCF[l2][(2 * 4 + v) * N + i], b);
-        dsum[v] = a + b;
+      for (int v = 0; v < 4; ++v) dsum[v] = a[v] + b[v];
+    };
+    // ---- phase 2: dQ/dt at the SPs and the Runge-Kutta stage; an SP's base
+    // state and lo planes come from global memory, the next SP's loads issued
+    // before this SP's stores (later stages update the state in place, so the
+    // compiler keeps loads behind earlier stores unless the program orders them
+    // first) ----
+    auto fetch = [&](int idx, T *bh, T *kl, T *bl) {
+      const size_t gi = ((size_t)e0 * NN + idx) * 4;
+#pragma unroll
+      for (int v = 0; v < 4; ++v) bh[v] = kl[v] = bl[v] = 0;
+      if (has_base) ld4((const T *)base.hi + gi, bh);
+      if constexpr (FF && LO) {
+        ld4((const T *)in.lo + gi, kl);
+        if (has_base) ld4((const T *)base.lo + gi, bl);
       }
     };
-    // ---- phase 2: dQ/dt at the SPs and the Runge-Kutta stage ----
-    if constexpr (MODE == MODE_RK && FF) {
-      // FP32: the base state and the lo planes of an SP come from global
-      // memory; the next SP's loads are issued before this SP's stores (later
-      // stages update the state in place, so the compiler keeps loads behind
-      // earlier stores unless the program orders them first)
-      auto fetch = [&](int idx, float *bh, float *kl, float *bl) {
-        const int l2 = idx / NN, sp = idx - l2 * NN;
+    T bh[4], kl[4], bl[4];
+    if (MODE == MODE_RK && (int)threadIdx.x < ne * NN) fetch(threadIdx.x, bh, kl, bl);
+    for (int idx = threadIdx.x; idx < ne * NN; idx += NT) {
+      T nbh[4], nkl[4], nbl[4];
+      if (MODE == MODE_RK && idx + NT < ne * NN) fetch(idx + NT, nbh, nkl, nbl);
+      const int l2 = idx / NN, sp = idx - l2 * NN;
+      const T iJ = ElemGeo<T, N, OTF>::inv_jac_at(md, sEF[l2], sEG + l2 * 8, sp, sXs[sp % N], sXs[sp / N]);
+      T dsum[4];
+      divergence(l2, sp, dsum);
+      if constexpr (MODE == MODE_RESIDUAL) {
         const size_t gi = ((size_t)(e0 + l2) * 4) * NN + sp;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          bh[v] = has_base ? ((const float *)base.hi)[gi + v * NN] : 0.0f;
-          kl[v] = LO ? ((const float *)in.lo)[gi + v * NN] : 0.0f;
-          bl[v] = (LO && has_base) ? ((const float *)base.lo)[gi + v * NN] : 0.0f;
-        }
-      };
-      float bh[4], kl[4], bl[4];
-      if ((int)threadIdx.x < ne * NN) fetch(threadIdx.x, bh, kl, bl);
-      for (int idx = threadIdx.x; idx < ne * NN; idx += NT) {
-        float nbh[4], nkl[4], nbl[4];
-        if (idx + NT < ne * NN) fetch(idx + NT, nbh, nkl, nbl);
-        const int l2 = idx / NN, sp = idx - l2 * NN;
-        const T iJ = ElemGeo<T, N, OTF>::inv_jac_t0(md, sEF[l2], sEG + l2 * 8, sp % N, sp / N);
-        const size_t gi = ((size_t)(e0 + l2) * 4) * NN + sp;
-        T dsum[4];
-        divergence(l2, sp, dsum);
-        float hv[4];
+        for (int v = 0; v < 4; ++v) Rout[gi + v * NN] = -(double)(dsum[v] * iJ);
+      } else {
+        const size_t gi = ((size_t)e0 * NN + idx) * 4;
+        T h[4], w[4], hn[4], ln[4];
+        ld4(sQ + 4 * idx, h);
+        if (w_in) ld4(w_in + gi, w);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-          const size_t ii = gi + v * NN;
-          const float R = -(float)(dsum[v] * iJ);
-          const float h = (float)sQ[l2][v][sp];
-          float inc = __fmul_rn((float)rk.bdt, R);
-          if constexpr (LO) {
-            const float l = kl[v];
-            if (has_base) inc = fmaf((float)rk.a0, (bh[v] - h) + (bl[v] - l), inc);
-            if (w_in) inc += (float)w_in[ii];
+          const T R = -(dsum[v] * iJ);
+          T inc = mul_rn(rk.bdt, R);
+          if constexpr (FF && LO) {
+            // double-float state: the increment added exactly (two-sum)
+            if (has_base) inc = fma(rk.a0, (bh[v] - h[v]) + (bl[v] - kl[v]), inc);
+            if (w_in) inc += w[v];
             float sum, err;
-            two_sum(h, inc, sum, err);
-            err += l;
-            const float H = sum + err;
-            ((float *)out.hi)[ii] = H;
-            ((float *)out.lo)[ii] = err - (H - sum);
-            hv[v] = H;
+            two_sum(h[v], inc, sum, err);
+            err += kl[v];
+            hn[v] = sum + err;
+            ln[v] = err - (hn[v] - sum);
           } else {
-            // single-float state: the stage result is rounded to float once
-            if (has_base) inc = fmaf((float)rk.a0, bh[v] - h, inc);
-            if (w_in) inc += (float)w_in[ii];
-            const float H = h + inc;
-            ((float *)out.hi)[ii] = H;
-            hv[v] = H;
+            // FP64, or a single-float state rounded to float once
+            if (has_base) inc = fma(rk.a0, bh[v] - h[v], inc);
+            if (w_in) inc += w[v];
+            hn[v] = h[v] + inc;
           }
-          if (w_out) w_out[ii] = (T)fmaf(-(float)rk.g, inc, (float)rk.ddt * R);
+          w[v] = FF ? fma(-rk.g, inc, rk.ddt * R) : mul_sub(rk.ddt, R, rk.g, inc);
         }
-        bad |= !physical(hv);
+        st4((T *)out.hi + gi, hn);
+        if constexpr (FF && LO) st4((T *)out.lo + gi, ln);
+        if (w_out) st4(w_out + gi, w);
+        bad |= !physical(hn);
+        st4(sQ + 4 * idx, hn);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-          sQ[l2][v][sp] = (T)hv[v];
           bh[v] = nbh[v];
           kl[v] = nkl[v];
           bl[v] = nbl[v];
         }
       }
-    } else
-    for (int idx = threadIdx.x; idx < ne * NN; idx += NT) {
-      const int l2 = idx / NN, sp = idx - l2 * NN;
-      const T iJ = ElemGeo<T, N, OTF>::inv_jac_t0(md, sEF[l2], sEG + l2 * 8, sp % N, sp / N);
-      const size_t gi = ((size_t)(e0 + l2) * 4) * NN + sp;
-      T dsum[4];
-      divergence(l2, sp, dsum);
-      if (MODE == MODE_RESIDUAL) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) Rout[gi + v * NN] = -(double)(dsum[v] * iJ);
-      } else if (!FF) {
-        double qn[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const size_t ii = gi + v * NN;
-          const double R = -(double)(dsum[v] * iJ);
-          const double qk = (double)sQ[l2][v][sp];
-          double inc = __dmul_rn((double)rk.bdt, R);
-          if (has_base) inc = fma((double)rk.a0, ((const double *)base.hi)[ii] - qk, inc);
-          if (w_in) inc += (double)w_in[ii];
-          qn[v] = qk + inc;
-          if (w_out) w_out[ii] = (T)mul_sub((double)rk.ddt, R, (double)rk.g, inc);
-        }
-        bad |= !physical(qn);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          ((double *)out.hi)[gi + v * NN] = qn[v];
-          sQ[l2][v][sp] = (T)qn[v];
-        }
-      } else {
-        float hv[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const size_t ii = gi + v * NN;
-          const float R = -(float)(dsum[v] * iJ);
-          const float h = (float)sQ[l2][v][sp];
-          float inc = __fmul_rn((float)rk.bdt, R);
-          if constexpr (LO) {
-            const float l = ((const float *)in.lo)[ii];
-            if (has_base)
-              inc = fmaf((float)rk.a0, (((const float *)base.hi)[ii] - h) + (((const float *)base.lo)[ii] - l), inc);
-            if (w_in) inc += (float)w_in[ii];
-            float sum, err;
-            two_sum(h, inc, sum, err);
-            err += l;
-            const float H = sum + err;
-            ((float *)out.hi)[ii] = H;
-            ((float *)out.lo)[ii] = err - (H - sum);
-            hv[v] = H;
-          } else {
-            // single-float state: the stage result is rounded to float once
-            if (has_base) inc = fmaf((float)rk.a0, ((const float *)base.hi)[ii] - h, inc);
-            if (w_in) inc += (float)w_in[ii];
-            const float H = h + inc;
-            ((float *)out.hi)[ii] = H;
-            hv[v] = H;
-          }
-          if (w_out) w_out[ii] = (T)fmaf(-(float)rk.g, inc, (float)rk.ddt * R);
-        }
-        bad |= !physical(hv);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) sQ[l2][v][sp] = (T)hv[v];
-      }
     }
     if (MODE == MODE_RK) {
       __syncthreads();
-      // ---- phase 3: face traces of the new state, one thread per SP line
-      // and variable (all the CTA's threads take part) ----
-      for (int q = threadIdx.x; q < 4 * C::LINES; q += NT) {
-        const int v = q / C::LINES, ln = q - v * C::LINES;
+      // ---- phase 3: face traces of the new state, one thread per end of an SP line ----
+      for (int q = threadIdx.x; q < 2 * C::LINES; q += NT) {
+        const int end = q / C::LINES, ln = q - end * C::LINES;
         const int l3 = ln / (2 * N), r3 = ln - l3 * 2 * N;
         const int d3 = r3 / N, m3 = r3 - d3 * N;
         if (l3 < ne) {
-          T *tr = (T *)md.TR + (size_t)(e0 + l3) * 16 * N;
-          const int fa = d3 == 0 ? 3 : 0, fb = d3 == 0 ? 1 : 2;
-          T a0 = 0, a1 = 0;
+          T a0[4] = {0, 0, 0, 0};
 #pragma unroll
           for (int k = 0; k < N; ++k) {
-            const T qk = d3 == 0 ? sQ[l3][v][m3 * N + k] : sQ[l3][v][k * N + m3];
-            a0 += qk * B.H0[k];
-            a1 += qk * B.H1[k];
+            T v[4];
+            ld4(sQ + 4 * (l3 * NN + (d3 == 0 ? m3 * N + k : k * N + m3)), v);
+            fma4(a0, end ? B.H1[k] : B.H0[k], v);
           }
-          tr[(fa * 4 + v) * N + m3] = a0;
-          tr[(fb * 4 + v) * N + m3] = a1;
+          const int f3 = d3 == 0 ? (end ? 1 : 3) : (end ? 2 : 0);
+          st4((T *)md.TR + ((size_t)(e0 + l3) * 4 + f3) * 4 * N + 4 * m3, a0);
         }
       }
     }
