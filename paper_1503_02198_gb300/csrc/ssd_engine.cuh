@@ -116,6 +116,13 @@ struct VolBasis {
   T Dm[N * (N + 1)];  // l'_{i+1/2}(X_k) [k][i]
   T H0[N], H1[N];     // h_k(0), h_k(1)
   T Xs[N], Xf[N + 1]; // solution and flux points
+  // Even and odd halves of the weights (FP64 path): the points are symmetric, so
+  // with sums and differences of mirrored values each half needs half of the
+  // multiplications.  Interpolation to FPs i and N - i: half (h_k +- h_{N-1-k}) at
+  // X_{i+1/2}, i = 1 .. N/2; derivative at SPs k and N - 1 - k: half (l'_i +- l'_{N-i})
+  // at X_k; for the middle point of an odd number the weight itself.
+  T He[(N / 2 + 1) * ((N + 1) / 2)], Ho[(N / 2 + 1) * ((N + 1) / 2)];
+  T De[((N + 1) / 2) * (N / 2 + 1)], Do[((N + 1) / 2) * (N / 2 + 1)];
   // the same weights duplicated into float pairs for packed FP32x2 FMAs
   float2 Hf2[(N + 1) * N], Dm2[N * (N + 1)], H02[N], H12[N];
 };
@@ -163,10 +170,17 @@ __device__ __forceinline__ T mul_sub(T a, T b, T c, T d) {
 }
 // a state value set that is physical: rho > 0, p > 0 and E finite.  With
 // rho > 0, p = (gamma - 1) (E - |m|^2 / (2 rho)) > 0 is 2 E rho > |m|^2,
-// which needs no division.
-template <typename T>
-__device__ __forceinline__ bool physical(const T *q) {
-  return q[0] > T(0) && T(2) * q[3] * q[0] - mul_add(q[1], q[1], q[2], q[2]) > T(0) && isfinite(q[3]);
+// which needs no division.  In FP64 only that test runs on the FP64 pipe: the
+// sign of rho and the exponent of E are tested as integers (a NaN rho fails the
+// second test).
+__device__ __forceinline__ bool physical(const float *q) {
+  return q[0] > 0.0f && 2.0f * q[3] * q[0] - mul_add(q[1], q[1], q[2], q[2]) > 0.0f && isfinite(q[3]);
+}
+__device__ __forceinline__ bool physical(const double *q) {
+  const int hi = __double2hiint(q[0]);
+  const bool rho = hi > 0 || (hi == 0 && __double2loint(q[0]) != 0);
+  const bool fin = (__double2hiint(q[3]) & 0x7ff00000) != 0x7ff00000;
+  return rho && fin && 2.0 * q[3] * q[0] - mul_add(q[1], q[1], q[2], q[2]) > 0.0;
 }
 
 // a product that is never fused into a later addition
@@ -208,6 +222,26 @@ __device__ __forceinline__ float recip_newton(float x) {
 template <typename T>
 __device__ __forceinline__ T recip(T x) {
   return recip_newton(x);
+}
+
+// Square root: the hardware's in FP32; in FP64 Goldschmidt's iteration (a
+// coupled Newton iteration for sqrt(x) and 1 / (2 sqrt(x))) from the hardware's
+// approximate reciprocal root, two steps and a last residual correction, ten
+// FP64 instructions, within an ulp or so; 0 for 0, NaN for negative x.
+__device__ __forceinline__ float root(float x) { return sqrtf(x); }
+__device__ __forceinline__ double root(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double g = x * y, h = 0.5 * y;
+  double r = fma(-g, h, 0.5);
+  g = fma(g, r, g);
+  h = fma(h, r, h);
+  r = fma(-g, h, 0.5);
+  g = fma(g, r, g);
+  h = fma(h, r, h);
+  g = fma(fma(-g, g, x), h, g);
+  // (x = 0: the reciprocal root is infinite)
+  return (__double2hiint(x) | __double2loint(x)) == 0 ? 0.0 : g;
 }
 
 // face f of an element: sign sigma_f with F~_end = sigma_f |S| F.n_out
@@ -577,7 +611,7 @@ struct ElemGeo {
     int ti = ((f & ~kIfaceBit) >> kZoneBits) - 1;
     if (!ssd_check(md, ti < md.nTab && (OTF || ti >= 0))) ti = 0;
     tab = OTF && ti < 0 ? nullptr : (const T *)md.geo + (size_t)ti * L::G;
-    if (OTF) {
+    if constexpr (OTF) {
       const float4 a = reinterpret_cast<const float4 *>(r)[0], b = reinterpret_cast<const float4 *>(r)[1];
       e1x = a.z, e1y = a.w, e3x = b.x, e3y = b.y, dx = b.z, dy = b.w;
     }
@@ -708,15 +742,25 @@ __device__ __forceinline__ void rusanov(const T *qL, const T *qR, T nx, T ny, T 
   const T gm1 = gamma - T(1);
   const T irL = recip(qL[0]), irR = recip(qR[0]);
   const T pL = pressure_ir(qL, irL, gm1), pR = pressure_ir(qR, irR, gm1);
-  T fL[4], fR[4];
-  normal_flux_ir(qL, irL, pL, nx, ny, vgn, fL);
-  normal_flux_ir(qR, irR, pR, nx, ny, vgn, fR);
   const T unL = mul_add(qL[1], nx, qL[2], ny) * irL, unR = mul_add(qR[1], nx, qR[2], ny) * irR;
-  const T lL = fabs(unL - vgn) + sqrt(gamma * pL * irL);
-  const T lR = fabs(unR - vgn) + sqrt(gamma * pR * irR);
+  const T lL = fabs(unL - vgn) + root(gamma * pL * irL);
+  const T lR = fabs(unR - vgn) + root(gamma * pR * irR);
   const T lam = lL > lR ? lL : lR;
+  if constexpr (std::is_same<T, double>::value) {
+    // the FP64 pipe's way: both sides' fluxes as one sum, the grid velocity
+    // taken off the normal velocities once (equal states still have no jump term)
+    const T wL = unL - vgn, wR = unR - vgn, ps = pL + pR, hl = T(-0.5) * lam;
+    const T t[4] = {fma(qL[0], wL, qR[0] * wR), fma(ps, nx, fma(qL[1], wL, qR[1] * wR)),
+                    fma(ps, ny, fma(qL[2], wL, qR[2] * wR)), fma(pL, unL, fma(pR, unR, fma(qL[3], wL, qR[3] * wR)))};
 #pragma unroll
-  for (int v = 0; v < 4; ++v) Fn[v] = mul_sub(T(0.5), fL[v] + fR[v], T(0.5) * lam, qR[v] - qL[v]);
+    for (int v = 0; v < 4; ++v) Fn[v] = fma(hl, qR[v] - qL[v], T(0.5) * t[v]);
+  } else {
+    T fL[4], fR[4];
+    normal_flux_ir(qL, irL, pL, nx, ny, vgn, fL);
+    normal_flux_ir(qR, irR, pR, nx, ny, vgn, fR);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) Fn[v] = mul_sub(T(0.5), fL[v] + fR[v], T(0.5) * lam, qR[v] - qL[v]);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1711,6 +1755,18 @@ __device__ __forceinline__ void point_flux(const T *q, T vx, T vy, T vg, T gm1, 
   f[3] = mul_sub(q[3] + p, un, vg, q[3]);
 }
 
+// point_flux() with V_g . a = 0
+template <typename T>
+__device__ __forceinline__ void point_flux_still(const T *q, T vx, T vy, T gm1, T *f) {
+  const T ir = recip(q[0]);
+  const T p = gm1 * (q[3] - T(0.5) * mul_add(q[1], q[1], q[2], q[2]) * ir);
+  const T un = mul_add(q[1], vx, q[2], vy) * ir;
+  f[0] = q[0] * un;
+  f[1] = fma(q[1], un, p * vx);
+  f[2] = fma(q[2], un, p * vy);
+  f[3] = (q[3] + p) * un;
+}
+
 // bounded wait by warp 0 only; the other warps wait at the barrier without issuing
 __device__ __forceinline__ bool cta_wait(uint64_t *bar, uint32_t parity, int polls = kWaitPolls) {
   bool ok = true;
@@ -2039,9 +2095,15 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
                                      (float(*)[8])(smem + C::O_TC));
     } else if (le < ne) {
       ElemGeo<T, N, OTF> G;
-      G.load_rec(md, e0 + le, sEF[le], sEG + le * 8, sZT);
       T mvx[N + 1], mvy[N + 1], mvg[N + 1];
-      G.line_metrics(d, mline, mvx, mvy, mvg);
+      const bool moving = FF || (sEF[le] & kZoneMask) != 0;
+      if (moving) {
+        G.load_rec(md, e0 + le, sEF[le], sEG + le * 8, sZT);
+        G.line_metrics(d, mline, mvx, mvy, mvg);
+      } else {
+        G.load_still(md, sEF[le], sEG + le * 8);
+        G.line_metrics_still(d, mline, mvx, mvy);
+      }
       if constexpr (FF) {
         // FP32: variables packed in pairs (rho, rho u), (rho v, E); every
         // interpolation and divergence FMA is a packed FP32x2 FMA
@@ -2115,52 +2177,96 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
           }
         }
       } else {
-      T q[4][N];
+        // FP64: bound by the FP64 pipe.  Values at mirrored points are taken as
+        // sums and differences (VolBasis): at N = 6 the interpolation of a line
+        // takes 25 instructions per variable instead of 30, its derivative 33
+        // instead of 42.  A pair of FPs (i, N - i) at a time: interpolation,
+        // fluxes, and their part of the divergence; on cells of the stationary
+        // zone without rotation and grid velocity.
+        constexpr int HK = (N + 1) / 2, HI = N / 2 + 1;
+        T qe[4][HK], qo[4][HK];
 #pragma unroll
-      for (int k = 0; k < N; ++k)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) q[v][k] = d == 0 ? sQ[le][(v) * NN + mline * N + k] : sQ[le][(v) * NN + k * N + mline];
-      T acc[4][N];
-#pragma unroll
-      for (int k = 0; k < N; ++k)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[v][k] = 0;
-#pragma unroll
-      for (int i = 0; i <= N; ++i) {
-        T f[4];
-        if (i == 0 || i == N) {
-          const int face = d == 0 ? (i == 0 ? 3 : 1) : (i == 0 ? 0 : 2);
-#pragma unroll
-          for (int v = 0; v < 4; ++v) f[v] = sCF[le][(face * 4 + v) * N + mline];
-        } else {
-          T qf[4];
+        for (int k = 0; k < HK; ++k)
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
-            T s = 0;
-#pragma unroll
-            for (int k = 0; k < N; ++k) s += q[v][k] * B.Hf[i * N + k];
-            qf[v] = s;
+            const int k2 = N - 1 - k;
+            const T x = d == 0 ? sQ[le][v * NN + mline * N + k] : sQ[le][v * NN + k * N + mline];
+            if (k2 == k) {
+              qe[v][k] = x;
+            } else {
+              const T y = d == 0 ? sQ[le][v * NN + mline * N + k2] : sQ[le][v * NN + k2 * N + mline];
+              qe[v][k] = x + y;
+              qo[v][k] = x - y;
+            }
           }
-          point_flux(qf, mvx[i], mvy[i], mvg[i], gm1, f);
+        T X[4][HK], Y[4][HK];  // divergence at SPs k and N - 1 - k: Y + X and Y - X
+#pragma unroll
+        for (int i = 0; i < HI; ++i) {
+          const int i2 = N - i;
+          T fe[4], fo[4];
+          if (i == 0) {
+            const int fa = d == 0 ? 3 : 0, fb = d == 0 ? 1 : 2;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              const T a = sCF[le][(fa * 4 + v) * N + mline], b = sCF[le][(fb * 4 + v) * N + mline];
+              fe[v] = a + b;
+              fo[v] = a - b;
+            }
+          } else {
+            T sa[4], sb2[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              T e = qe[v][0] * B.He[i * HK];
+#pragma unroll
+              for (int k = 1; k < HK; ++k) e = fma(qe[v][k], B.He[i * HK + k], e);
+              if (i2 == i) {
+                sa[v] = e;
+              } else {
+                T o = qo[v][0] * B.Ho[i * HK];
+#pragma unroll
+                for (int k = 1; k < N / 2; ++k) o = fma(qo[v][k], B.Ho[i * HK + k], o);
+                sa[v] = e + o;
+                sb2[v] = e - o;
+              }
+            }
+            T f[4], f2v[4];
+            if (moving) {
+              point_flux(sa, mvx[i], mvy[i], mvg[i], gm1, f);
+              if (i2 != i) point_flux(sb2, mvx[i2], mvy[i2], mvg[i2], gm1, f2v);
+            } else {
+              point_flux_still(sa, mvx[i], mvy[i], gm1, f);
+              if (i2 != i) point_flux_still(sb2, mvx[i2], mvy[i2], gm1, f2v);
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              fe[v] = i2 == i ? f[v] : f[v] + f2v[v];
+              fo[v] = i2 == i ? T(0) : f[v] - f2v[v];
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < HK; ++k)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              if (2 * k != N - 1)
+                X[v][k] = i == 0 ? B.De[k * HI] * fe[v] : fma(B.De[k * HI + i], fe[v], X[v][k]);
+              if (i2 != i) Y[v][k] = i == 0 ? B.Do[k * HI] * fo[v] : fma(B.Do[k * HI + i], fo[v], Y[v][k]);
+            }
         }
+        T *o = (d == 0 ? sRF[le] : sRG[le]);
 #pragma unroll
-        for (int k = 0; k < N; ++k) {
-          const T w = B.Dm[k * (N + 1) + i];
+        for (int k = 0; k < HK; ++k)
 #pragma unroll
-          for (int v = 0; v < 4; ++v) acc[v][k] += w * f[v];
-        }
-      }
-      if (d == 0) {
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) sRF[le][(v) * NN + mline * N + k] = acc[v][k];
-      } else {
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) sRG[le][(v) * NN + k * N + mline] = acc[v][k];
-      }
+          for (int v = 0; v < 4; ++v) {
+            const int k2 = N - 1 - k;
+            const int p1 = v * NN + (d == 0 ? mline * N + k : k * N + mline);
+            const int p2 = v * NN + (d == 0 ? mline * N + k2 : k2 * N + mline);
+            if (k2 == k) {
+              o[p1] = Y[v][k];
+            } else {
+              o[p1] = Y[v][k] + X[v][k];
+              o[p2] = Y[v][k] - X[v][k];
+            }
+          }
       }
     }
     // the single-buffered part (state lo, base state) must have landed too
@@ -2189,11 +2295,13 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
         const double(*sW)[4 * NN] = (const double(*)[4 * NN])(smem + C::O_AUX);
         double *qo = (double *)va.out.hi;
         double qn[4];
+        const double c = -(double)va.rk.bdt * (double)iJ;
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-          const double R = -(double)((sRF[l2][(v) * NN + sp] + sRG[l2][(v) * NN + sp]) * iJ);
+          const double div = (double)(sRF[l2][(v) * NN + sp] + sRG[l2][(v) * NN + sp]);
+          const double R = va.w_out ? -div * (double)iJ : 0.0;
           const double qk = (double)sQ[l2][(v) * NN + sp];
-          double inc = __dmul_rn((double)va.rk.bdt, R);
+          double inc = __dmul_rn(c, div);
           if (use_base) inc = fma((double)va.rk.a0, sN[l2][(v) * NN + sp] - qk, inc);
           if (AUX) inc += sW[l2][(v) * NN + sp];
           qn[v] = qk + inc;
@@ -2514,6 +2622,20 @@ struct EngineImpl : Engine {
       mb.cden[k] = hb.cden[k];
     }
     for (int k = 0; k <= N; ++k) vb.Xf[k] = (T)hb.Xf[k];
+    for (int i = 0; i <= N / 2; ++i)
+      for (int k = 0; k < (N + 1) / 2; ++k) {
+        const bool mid = 2 * k == N - 1;  // the SP that mirrors itself
+        const double a = hb.Hf[i * N + k], b = hb.Hf[i * N + N - 1 - k];
+        vb.He[i * ((N + 1) / 2) + k] = (T)(mid ? a : 0.5 * (a + b));
+        vb.Ho[i * ((N + 1) / 2) + k] = (T)(mid ? 0.0 : 0.5 * (a - b));
+      }
+    for (int k = 0; k < (N + 1) / 2; ++k)
+      for (int i = 0; i <= N / 2; ++i) {
+        const bool mid = 2 * i == N;  // the FP that mirrors itself
+        const double a = hb.Dm[k * (N + 1) + i], b = hb.Dm[k * (N + 1) + N - i];
+        vb.De[k * (N / 2 + 1) + i] = (T)(mid ? a : 0.5 * (a + b));
+        vb.Do[k * (N / 2 + 1) + i] = (T)(mid ? 0.0 : 0.5 * (a - b));
+      }
     for (int k = 0; k < (N + 1) * N; ++k) {
       vb.Hf2[k] = make_float2((float)hb.Hf[k], (float)hb.Hf[k]);
       vb.Dm2[k] = make_float2((float)hb.Dm[k], (float)hb.Dm[k]);

@@ -211,17 +211,6 @@ __device__ __forceinline__ void rusanov2(const float2 *q, const float2 *n, float
     F[v] = f2_fma(f2(-0.5f), f2_add(f[0][v], f[1][v]), f2_mul(hl, f2_sub(n[v], q[v])));
 }
 
-// point_flux() with V_g . a = 0
-__device__ __forceinline__ void point_flux_still(const float *q, float vx, float vy, float gm1, float *f) {
-  const float ir = recip(q[0]);
-  const float p = gm1 * (q[3] - 0.5f * mul_add(q[1], q[1], q[2], q[2]) * ir);
-  const float un = mul_add(q[1], vx, q[2], vy) * ir;
-  f[0] = q[0] * un;
-  f[1] = fmaf(q[1], un, p * vx);
-  f[2] = fmaf(q[2], un, p * vy);
-  f[3] = (q[3] + p) * un;
-}
-
 // Shared-memory layout: two stages of a tile's state hi (padded element
 // stride, as k_volume's), cell records and flags; three slots of face records
 // (a tile's arrive one tile ahead of its state, since they name the traces to

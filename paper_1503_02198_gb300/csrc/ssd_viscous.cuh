@@ -74,6 +74,38 @@ __device__ __forceinline__ void viscous_flux(const T *q, const T *qx, const T *q
   G[3] = -fma(u, txy, mul_add(v, tyy, kr, Ty));
 }
 
+// The FP64 pipe's way to the same fluxes through a vector (nx, ny): one
+// reciprocal, the stress and heat flux taken along the vector first (three
+// products where F and G are formed in full: six), no zero component.  Adds the
+// viscous flux to f; u, v, ke, pr as viscous_flux forms them.
+__device__ __forceinline__ void add_viscous_along(const double *qx, const double *qy, double ir, double u, double v,
+                                                  double ke, double pr, const MeshDev &md, double nx, double ny,
+                                                  double kr, double *f) {
+  const double ux = fma(-u, qx[0], qx[1]) * ir, uy = fma(-u, qy[0], qy[1]) * ir;
+  const double vx = fma(-v, qx[0], qx[2]) * ir, vy = fma(-v, qy[0], qy[2]) * ir;
+  const double px = md.gm1 * fma(ke, qx[0], fma(-v, qx[2], fma(-u, qx[1], qx[3])));
+  const double py = md.gm1 * fma(ke, qy[0], fma(-v, qy[2], fma(-u, qy[1], qy[3])));
+  const double Tx = fma(-pr, qx[0], px) * ir, Ty = fma(-pr, qy[0], py) * ir;
+  const double l = (-2.0 / 3.0 * md.mu) * (ux + vy), m2 = 2.0 * md.mu;
+  const double txx = fma(m2, ux, l), tyy = fma(m2, vy, l), txy = md.mu * (uy + vx);
+  const double tx = fma(txx, nx, txy * ny), ty = fma(txy, nx, tyy * ny), qn = fma(Tx, nx, Ty * ny);
+  f[1] -= tx;
+  f[2] -= ty;
+  f[3] = fma(-u, tx, fma(-v, ty, fma(-kr, qn, f[3])));
+}
+
+// inviscid ALE and viscous flux through (nx, ny) with vgn = V_g . (nx, ny)
+__device__ __forceinline__ void total_flux(const double *q, const double *g8, const MeshDev &md, double nx, double ny,
+                                           double vgn, double *f) {
+  const double ir = recip(q[0]), u = q[1] * ir, v = q[2] * ir, ke = 0.5 * fma(u, u, v * v);
+  const double p = md.gm1 * fma(-ke, q[0], q[3]), un = fma(u, nx, v * ny), w = un - vgn;
+  f[0] = q[0] * w;
+  f[1] = fma(q[1], w, p * nx);
+  f[2] = fma(q[2], w, p * ny);
+  f[3] = fma(q[3], w, p * un);
+  add_viscous_along(g8, g8 + 4, ir, u, v, ke, p * ir, md, nx, ny, md.kcR, f);
+}
+
 // ---- state conversion and traces ----------------------------------------------
 
 // FP64 state [E][4][N^2] -> the points layout (a double-float pair, a float or a
@@ -366,10 +398,17 @@ __global__ void __launch_bounds__(GradCfg<T, N>::THREADS) k_grad_trace(Src src, 
 template <typename T>
 __device__ __forceinline__ void viscous_normal(const T *q, const T *g8, T nx, T ny, const MeshDev &md, T *fn,
                                                bool conduct = true) {
-  T F[4], G[4];
-  viscous_flux(q, g8, g8 + 4, md, F, G, conduct);
+  if constexpr (std::is_same<T, double>::value) {
+    const T ir = recip(q[0]), u = q[1] * ir, v = q[2] * ir, ke = T(0.5) * fma(u, u, v * v);
+    const T pr = md.gm1 * fma(-ke, q[0], q[3]) * ir;
+    fn[0] = fn[1] = fn[2] = fn[3] = T(0);
+    add_viscous_along(g8, g8 + 4, ir, u, v, ke, pr, md, nx, ny, conduct ? md.kcR : 0.0, fn);
+  } else {
+    T F[4], G[4];
+    viscous_flux(q, g8, g8 + 4, md, F, G, conduct);
 #pragma unroll
-  for (int v = 0; v < 4; ++v) fn[v] = mul_add(F[v], nx, G[v], ny);
+    for (int v = 0; v < 4; ++v) fn[v] = mul_add(F[v], nx, G[v], ny);
+  }
 }
 
 template <typename T, int N>
@@ -611,14 +650,18 @@ __global__ void __launch_bounds__(VisVolCfg<T, N>::THREADS, VisVolCfg<T, N>::MIN
       }
       T vx, vy, vg;
       G.fp_at(d, fi, m, sXf[fi], sXs[m], vx, vy, vg);
-      const T p = pressure_of(qf, gm1);
-      T f[4], Fv[4], Gv[4];
-      normal_flux(qf, p, vx, vy, vg, f);
-      viscous_flux(qf, g8, g8 + 4, md, Fv, Gv);
-      T *o = sFl + ((le * 2 + d) * N + m) * C::LS + (fi - 1) * 4;
+      T f[4];
+      if constexpr (std::is_same<T, double>::value) {
+        total_flux(qf, g8, md, vx, vy, vg, f);
+      } else {
+        const T p = pressure_of(qf, gm1);
+        T Fv[4], Gv[4];
+        normal_flux(qf, p, vx, vy, vg, f);
+        viscous_flux(qf, g8, g8 + 4, md, Fv, Gv);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) f[v] = fma(vx, Fv[v], fma(vy, Gv[v], f[v]));
-      st4(o, f);
+        for (int v = 0; v < 4; ++v) f[v] = fma(vx, Fv[v], fma(vy, Gv[v], f[v]));
+      }
+      st4(sFl + ((le * 2 + d) * N + m) * C::LS + (fi - 1) * 4, f);
     }
     __syncthreads();
     // (RF + RG)[v] at SP sp = (i, j) of element l2: each direction's
