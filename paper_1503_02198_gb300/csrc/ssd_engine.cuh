@@ -2866,7 +2866,7 @@ struct EngineImpl : Engine {
       const int nmort = fuse_faces_mortar ? (md.nM + C::EPB - 1) / C::EPB : 0;
       const int nblk = fuse_faces_mortar ? nmort + (md.nB * N + C::THREADS - 1) / C::THREADS : 0;
       launch_pdl(k_stage<N, MODE, AUX, LO>, std::min(ntiles, grid), C::THREADS, C::SMEM, s, md, vol_args(in, base, out, R, rk), ntiles,
-                 early_tiles, nmort, nblk, ahead_stage(ntiles, grid));
+                 early_tiles, nmort, nblk, ahead_stage(ntiles, grid), (int)((const char *)md.TR > (const char *)md.TRo));
     }
   }
 
