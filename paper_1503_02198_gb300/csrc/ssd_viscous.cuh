@@ -208,11 +208,12 @@ __global__ void k_faces_cq(MeshDev md) {
 // ---- gradients ---------------------------------------------------------------
 
 // Elements per block of the viscous kernels (two threads per SP line pair:
-// 2 N threads per element): chosen so that a block is whole warps.
+// 2 N threads per element).  FP32 N = 5: 161 us a step with 4, 163 with 8 and 16
+// (20,096 cells: about one and a half tiles per CTA slot, so small tiles end together).
 template <typename T, int N>
 struct VisCfg {
   static constexpr bool F = sizeof(T) == 4;
-  static constexpr int EPB = N == 3 ? 16 : (N == 4 ? 8 : (N == 5 ? (F ? 16 : 8) : (F ? 8 : 4)));
+  static constexpr int EPB = N == 3 ? 16 : (N == 4 ? 8 : (N == 5 ? (F ? 4 : 8) : (F ? 8 : 4)));
   static constexpr int THREADS = EPB * 2 * N;
   // resident blocks per SM the register budget is set for: about 16 warps
   static constexpr int MINB = 16 / ((THREADS + 31) / 32) > 0 ? 16 / ((THREADS + 31) / 32) : 1;
@@ -498,7 +499,9 @@ __global__ void k_faces_visc(MeshDev md) {
 // threads per element, so that a CTA holds few elements and many threads.
 template <typename T, int N>
 struct VisVolCfg {
-  static constexpr int EPB = N == 3 ? 16 : (N == 4 ? 8 : 4);
+  // elements per tile (FP32 N = 4: 149 us a step with 4, 151 with 8, 163 with 16
+  // on 14,752 cells, five stages; N = 5: 163 with 4, 172 with 8 on 20,096 cells)
+  static constexpr int EPB = N == 3 ? 16 : (N == 4 && sizeof(T) == 8 ? 8 : 4);
   static constexpr int NN = N * N, LINES = EPB * 2 * N, THREADS = LINES * (N - 1);
   static constexpr int QE = 4 * NN * (int)sizeof(T), GE = 8 * NN * (int)sizeof(T), CE = 16 * N * (int)sizeof(T);
   static constexpr int GEE = 8 * (int)sizeof(T);  // bilinear cell record
