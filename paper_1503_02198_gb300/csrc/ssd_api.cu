@@ -1087,11 +1087,12 @@ int sd_set_state(sd_handle *h, const double *Q, int on_device) {
     // the conversion reads the caller's buffer itself when the device can
     // address it (pinned host memory), else a staged copy
     const double *src = on_device ? Q : (const double *)mapped_host(Q);
+    const bool host = !on_device && src;
     if (!src) {
       e = cudaMemcpyAsync(h->stage, Q, state_bytes(h), cudaMemcpyHostToDevice, h->stream);
       src = h->stage;
     }
-    if (!e) h->eng->set_state(h->md, src, h->stream);
+    if (!e) h->eng->set_state(h->md, src, host, h->stream);
     if (!e) e = cudaGetLastError();
   }
   if (!e && !on_device) e = cudaStreamSynchronize(h->stream);  // caller may reuse Q at once
@@ -1110,7 +1111,7 @@ int sd_get_state(sd_handle *h, double *Q, int on_device) {
     // written straight into a pinned host buffer, else staged and copied
     double *direct = on_device ? Q : (double *)mapped_host(Q);
     double *dst = direct ? direct : h->stage;
-    h->eng->get_state(h->md, dst, h->stream);
+    h->eng->get_state(h->md, dst, !on_device && direct, h->stream);
     e = cudaGetLastError();
     if (!e && !direct) e = cudaMemcpyAsync(Q, dst, state_bytes(h), cudaMemcpyDeviceToHost, h->stream);
   }

@@ -18,10 +18,11 @@
 //                   with its R node angles -> mortars, (o, s) of each mortar
 //                   against its L and R face (Eq. xz), face ranges, into the
 //                   stage's own clock record and mortar table.  Off the
-//                   critical path: stages 1.. are merged beside stage 0's
-//                   kernels, and stage 0 of the next step beside stage 1's
-//                   (k_clock_merge: the same for one stage, e.g. a residual)
-// Per stage:
+//                   critical path: the stages of the next step are merged
+//                   beside this one's (k_clock_merge: the same for one stage,
+//                   e.g. a residual)
+// Per stage, FP32 forms on Euler meshes: k_stage (ssd_stage.cuh) does all of
+// the following in one launch.  Viscous meshes: ssd_viscous.cuh.  Else:
 //   k_faces         one launch for every face point: conforming and periodic
 //                   faces (Rusanov common flux), then boundary faces (wall,
 //                   slip, inlet, outlet, adiabatic: Rusanov through a ghost state)
@@ -1604,6 +1605,38 @@ static __global__ void k_join(const float *__restrict__ hi, const float *__restr
   Q[i] = lo ? (double)hi[i] + (double)lo[i] : (double)hi[i];
 }
 
+// Word of the state value that is number i of [E][4][N][N], in another layout.
+template <int N, int LAY>
+__device__ __forceinline__ size_t state_word(size_t i) {
+  constexpr unsigned NN = N * N;
+  const size_t e = i / (4 * NN);
+  const unsigned r = (unsigned)(i - e * 4 * NN), v = r / NN, sp = r - v * NN;
+  return e * 4 * NN + (LAY == LAY_POINTS ? 4 * sp + v : (v >> 1) * 2 * NN + 2 * sp + (v & 1));
+}
+
+// The conversions for a state in host memory: one value per thread, so that the
+// host side is read and written in unbroken runs (by pairs of variables the
+// runs are N^2 values long and the link gives 187 GB/s instead of 208 on a
+// 284 MB state); the device side is scattered within an element.
+template <typename T, int N, int LAY>
+__global__ void k_split_linear(const double *__restrict__ Q, T *hi, T *lo, size_t n) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double x = Q[i];
+  const T h = (T)x;
+  const size_t w = state_word<N, LAY>(i);
+  hi[w] = h;
+  if (lo) lo[w] = (T)(x - (double)h);
+}
+
+template <typename T, int N, int LAY>
+__global__ void k_join_linear(const T *__restrict__ hi, const T *__restrict__ lo, double *Q, size_t n) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const size_t w = state_word<N, LAY>(i);
+  Q[i] = lo ? (double)hi[w] + (double)lo[w] : (double)hi[w];
+}
+
 // face traces [E][4][4][N] of a state (compute-precision values)
 template <typename T, int N>
 __global__ void k_trace(MeshDev md, const T *__restrict__ Q) {
@@ -2566,7 +2599,13 @@ struct EngineImpl : Engine {
   StatePtr A() const override { return StatePtr{sA[0], sA[1]}; }
   StatePtr B() const override { return StatePtr{sB[0], sB[1]}; }
 
-  void set_state(const MeshDev &md, const double *Q, cudaStream_t s) override {
+  void set_state(const MeshDev &md, const double *Q, bool host, cudaStream_t s) override {
+    if (host && (md.frec || md.viscous)) {
+      const unsigned nb = (unsigned)((nval + 255) / 256);
+      if (md.viscous) k_split_linear<T, N, LAY_POINTS><<<nb, 256, 0, s>>>(Q, (T *)sA[0], (T *)sA[1], nval);
+      else k_split_linear<T, N, LAY_PAIRS><<<nb, 256, 0, s>>>(Q, (T *)sA[0], (T *)sA[1], nval);
+      return;
+    }
     if constexpr (OTF) {
       if (md.frec) {
         const int n = (int)(nval / 2);
@@ -2586,7 +2625,13 @@ struct EngineImpl : Engine {
     else
       cudaMemcpyAsync(sA[0], Q, sizeof(double) * nval, cudaMemcpyDeviceToDevice, s);
   }
-  void get_state(const MeshDev &md, double *Q, cudaStream_t s) override {
+  void get_state(const MeshDev &md, double *Q, bool host, cudaStream_t s) override {
+    if (host && (md.frec || md.viscous)) {
+      const unsigned nb = (unsigned)((nval + 255) / 256);
+      if (md.viscous) k_join_linear<T, N, LAY_POINTS><<<nb, 256, 0, s>>>((const T *)sA[0], (const T *)sA[1], Q, nval);
+      else k_join_linear<T, N, LAY_PAIRS><<<nb, 256, 0, s>>>((const T *)sA[0], (const T *)sA[1], Q, nval);
+      return;
+    }
     if constexpr (OTF) {
       if (md.frec) {
         const int n = (int)(nval / 2);

@@ -244,8 +244,9 @@ struct Engine {
   virtual StatePtr A() const = 0;
   virtual StatePtr B() const = 0;
   // copy an FP64 state (device memory) into A, or A out as FP64 (device memory)
-  virtual void set_state(const MeshDev &md, const double *Q, cudaStream_t s) = 0;
-  virtual void get_state(const MeshDev &md, double *Q, cudaStream_t s) = 0;
+  // (host: Q is mapped host memory)
+  virtual void set_state(const MeshDev &md, const double *Q, bool host, cudaStream_t s) = 0;
+  virtual void get_state(const MeshDev &md, double *Q, bool host, cudaStream_t s) = 0;
   // upload basis constants, compute the t = 0 metrics
   virtual cudaError_t init(const HostBasis &hb, const MeshDev &md, cudaStream_t s) = 0;
   // face traces of a state
