@@ -95,24 +95,23 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# DRAM bytes (read + write) per launch of the FP32 volume kernel on this
+# DRAM bytes (read + write) per launch of the FP32 stage kernel on this
 # workload (mean of the three stage launches of one step), from one ncu
 # capture of dram__bytes_read.sum + dram__bytes_write.sum; valid only for the
-# kernel source it was taken on: SHA-256 of the engine text that k_volume is
-# built from (its helpers, the ElemGeo metrics and VolCfg, from the start of
-# the engine header through the end of k_volume); otherwise null.
-PROFILED_TRAFFIC = {"bytes": (389.3e6 + 329.1e6 + 673.7e6 + 330.8e6 + 673.6e6 + 329.5e6) / 3,
-                    "kernel_sha256": "08c0c761564d75e3ec7ff3855a811e014f811251ac5c17f80dc192a794330087"}
+# kernel source it was taken on: SHA-256 of the engine text that k_stage is
+# built from (its helpers and the ElemGeo metrics, from the start of the engine
+# header up to the viscous path, and ssd_stage.cuh); otherwise null.
+PROFILED_TRAFFIC = {"bytes": 0.0, "kernel_sha256": ""}
 
 
 def volume_kernel_source():
-    path = os.path.join(ROOT, "paper_1503_02198_gb300", "csrc", "ssd_engine.cuh")
+    csrc = os.path.join(ROOT, "paper_1503_02198_gb300", "csrc")
     try:
-        text = open(path, encoding="utf-8").read()
+        text = open(os.path.join(csrc, "ssd_engine.cuh"), encoding="utf-8").read()
+        stage = open(os.path.join(csrc, "ssd_stage.cuh"), encoding="utf-8").read()
     except OSError:
         return None
-    d = text.index('#include "ssd_viscous.cuh"')
-    return text[:d]
+    return text[:text.index('#include "ssd_viscous.cuh"')] + stage
 
 
 def profiled_traffic():
@@ -124,15 +123,16 @@ def profiled_traffic():
     return PROFILED_TRAFFIC["bytes"] if h == PROFILED_TRAFFIC["kernel_sha256"] else None
 
 
-def volume_bytes_per_element(N, w_c, w_s=8):
+def volume_bytes_per_element(N, w_c, w_s=8, stage_kernel=False):
     """Algorithmic bytes one volume launch moves per element (see design
     notes): state read + write (w_s bytes per value: 8 for the FP64 or
     double-float state, 4 for FP32 state storage), the Runge-Kutta base read
-    on two of the three stages, the common-flux read and the new traces
-    written (16 N values each in the compute word), 4 corner nodes (16 B each)
-    and the zone tag."""
+    on two of the three stages, the common-flux read (stage_kernel: the
+    neighbours' traces) and the new traces written (16 N values each in the
+    compute word), 4 corner nodes (16 B each; stage_kernel: the cell record
+    and 4 face records) and the zone tag."""
     state = 4 * N * N * w_s
-    return state * (2 + 2.0 / 3.0) + 2 * 16 * N * w_c + 4 * 16 + 4
+    return state * (2 + 2.0 / 3.0) + 2 * 16 * N * w_c + (32 + 4 * 16 if stage_kernel else 4 * 16) + 4
 
 
 def volume_flops_per_element(N):
@@ -156,7 +156,9 @@ def interface_fraction(prof):
     "interface" time (Tables 3-10): the stage clock and mortar merge and the
     mortar projections with their common flux, each timed as its own launch
     by sd_profile_step (per stage; three stages a step; the sum over each
-    face's mortars runs inside the volume kernel and is not counted)."""
+    face's mortars runs inside the volume kernel and is not counted; in a
+    captured step the merges run beside it and, on the FP32 Euler path, the
+    mortars inside the stage launch)."""
     return (prof["merge"] + prof["mortar"]) * 3 / prof["step"]
 
 
@@ -688,12 +690,12 @@ def main():
             Q3 = s3.sd_get_state()
             fp32s["rel_l2_vs_fp64"] = float(np.sqrt(np.sum((Q3 - Q64) ** 2) / np.sum(Q64 ** 2)))
         prof3 = s3.sd_profile_step(dt, reps=5)
-        vb3 = volume_bytes_per_element(N, 4, 4) * s3.E
+        vb3 = volume_bytes_per_element(N, 4, 4, True) * s3.E
         ach3 = vb3 / (prof3["volume"] * 1e-3) / 1e9
         pk, _ = _peaks()
         fp32s["kernel_ms"] = prof3
         fp32s["roofline"] = {"bound": "hbm", "achieved": ach3, "peak": pk, "unit": "GB/s", "frac": ach3 / pk,
-                             "kernel": "k_volume", "algorithmic_bytes_per_launch": vb3}
+                             "kernel": "k_stage", "algorithmic_bytes_per_launch": vb3}
         s3.close()
 
     # the FP32 form with the volume contractions on the tensor cores (3xTF32):
@@ -727,7 +729,8 @@ def main():
     prof = solver.sd_profile_step(dt, reps=5)
     w_c = 8 if prec == ssd.SD_PREC_FP64 else 4
     E = solver.E
-    vol_bytes = volume_bytes_per_element(N, w_c, 4 if prec == ssd.SD_PREC_FP32S else 8) * E
+    stage_kernel = prec in (ssd.SD_PREC_FP32, ssd.SD_PREC_FP32S) and not w.params.viscous
+    vol_bytes = volume_bytes_per_element(N, w_c, 4 if prec == ssd.SD_PREC_FP32S else 8, stage_kernel) * E
     peak, peak_src = _peaks()
     achieved = vol_bytes / (prof["volume"] * 1e-3) / 1e9
     traffic = profiled_traffic() if (args.workload == "rotor_n6" and prec == ssd.SD_PREC_FP32) else None
@@ -735,7 +738,7 @@ def main():
                 "traffic": traffic,
                 "traffic_source": ("stored ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of this "
                                    "kernel source, not a measurement of this run") if traffic else None,
-                "kernel": "k_volume", "peak_source": peak_src + " hbm_gbs (burst)",
+                "kernel": "k_stage" if stage_kernel else "k_volume", "peak_source": peak_src + " hbm_gbs (burst)",
                 "algorithmic_bytes_per_launch": vol_bytes}
     try:
         fp32_peak = solver.sd_fma_peak(ssd.SD_PREC_FP32)
@@ -818,8 +821,7 @@ def main():
             "cpu_baseline": cpu,
             "e2e": e2e,
             "clocks": clocks,
-            "gpu_launches": launches_per_step(w.mesh, w.params.viscous,
-                                              prec in (ssd.SD_PREC_FP32, ssd.SD_PREC_FP32S)) * args.steps,
+            "gpu_launches": launches_per_step(w.mesh, w.params.viscous, stage_kernel) * args.steps,
         }
         print(json.dumps(line))
     if world > 1:

@@ -21,8 +21,8 @@
 // bandwidth 69 %, issue 49 %, DRAM 1.03 GB per later stage (4.9 TB/s); barrier,
 // wait and shared-load stalls 1.3 each per issue with 15 warps per SM.  A step
 // took 703 us with the face pass (48 us) and the volume kernel (180 us) apart
-// and takes 613 us here (float state, 123,450 cells: 322 -> 289 us; 31,509 cells
-// at N = 3: 72 -> 53 us).
+// and takes 598 us here (float state, 123,450 cells: 322 -> 282 us; 31,509 cells
+// at N = 3: 72 -> 53 us; 6,016 cells at N = 4: 39 -> 29 us).
 #pragma once
 
 namespace ssd {
@@ -215,7 +215,7 @@ __device__ __forceinline__ void rusanov2(const float2 *q, const float2 *n, float
 // stride, as k_volume's), cell records and flags; three slots of face records
 // (a tile's arrive one tile ahead of its state, since they name the traces to
 // load); the Runge-Kutta inputs; the two directions' divergences; barriers;
-// the zone table.  No common-flux tile: 30 to 35 KB instead of 42 KB at N = 6.
+// the zone table; each thread's prefetched end points.  44 KB at N = 6.
 template <int N, bool AUX, bool LO>
 struct StageCfg {
   using V = VolCfg<float, N, true, AUX, LO>;
