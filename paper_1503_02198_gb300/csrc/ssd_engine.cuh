@@ -161,6 +161,16 @@ struct GeoLayout {
 // of such a sum may be fused, and two kernels that inline the same expression
 // (a single case's kernel and a batch class's) may choose differently and
 // differ in the last bit; written out, every kernel computes the same bits.
+// The same goes for a single product that is summed: the metric vectors of
+// stationary cells, x + u d, were fused at N = 6 and left apart at N = 3 to 5,
+// and one cell in twenty of a mesh with skewed cells got other last bits than
+// from the general form.  Such sums are an explicit fma() below, and a product
+// that is used both in a sum and elsewhere (the pressure) is rounded once by
+// mul_rn().
+// a product that is never fused into a later addition
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 template <typename T>
 __device__ __forceinline__ T mul_add(T a, T b, T c, T d) {
   return fma(a, b, c * d);
@@ -183,10 +193,6 @@ __device__ __forceinline__ bool physical(const double *q) {
   const bool fin = (__double2hiint(q[3]) & 0x7ff00000) != 0x7ff00000;
   return rho && fin && 2.0 * q[3] * q[0] - mul_add(q[1], q[1], q[2], q[2]) > 0.0;
 }
-
-// a product that is never fused into a later addition
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
 // a parameter in the compute type, taken from its float copy on the FP32
 // path so that no FP64 instruction runs there
@@ -521,12 +527,12 @@ struct ElemGeo {
   __device__ __forceinline__ void xi_fp(int i, int j, T &vx, T &vy, T &g) const {
     if (OTF && tab == nullptr) {
       const T xi = cVB<T, N>.Xf[i], eta = cVB<T, N>.Xs[j];
-      const T xe = e3x + xi * dx, ye = e3y + xi * dy;
+      const T xe = fma(xi, dx, e3x), ye = fma(xi, dy, e3y);
       vx = ye;
       vy = -xe;
       g = T(0);
       if (om != T(0)) {
-        const T px = x0 + xi * e1x + eta * xe, py = y0 + xi * e1y + eta * ye;
+        const T px = fma(eta, xe, fma(xi, e1x, x0)), py = fma(eta, ye, fma(xi, e1y, y0));
         g = om * mul_sub(px, vy, py, vx);
       }
     } else {
@@ -541,12 +547,12 @@ struct ElemGeo {
   __device__ __forceinline__ void eta_fp(int i, int l, T &vx, T &vy, T &g) const {
     if (OTF && tab == nullptr) {
       const T xi = cVB<T, N>.Xs[i], eta = cVB<T, N>.Xf[l];
-      const T xx = e1x + eta * dx, yx = e1y + eta * dy;
+      const T xx = fma(eta, dx, e1x), yx = fma(eta, dy, e1y);
       vx = -yx;
       vy = xx;
       g = T(0);
       if (om != T(0)) {
-        const T px = x0 + eta * e3x + xi * xx, py = y0 + eta * e3y + xi * yx;
+        const T px = fma(xi, xx, fma(eta, e3x, x0)), py = fma(xi, yx, fma(eta, e3y, y0));
         g = om * mul_sub(px, vy, py, vx);
       }
     } else {
@@ -561,12 +567,12 @@ struct ElemGeo {
   // the point's coordinates u = X_{i+1/2}, w = X_m at hand
   __device__ __forceinline__ void fp_at(int d, int i, int m, T u, T w, T &vx, T &vy, T &g) const {
     if (OTF && tab == nullptr) {
-      const T tx = (d == 0 ? e3x : e1x) + u * dx, ty = (d == 0 ? e3y : e1y) + u * dy;
+      const T tx = fma(u, dx, d == 0 ? e3x : e1x), ty = fma(u, dy, d == 0 ? e3y : e1y);
       vx = d == 0 ? ty : -ty;
       vy = d == 0 ? -tx : tx;
       g = T(0);
       if (om != T(0)) {
-        const T px = x0 + u * (d == 0 ? e1x : e3x) + w * tx, py = y0 + u * (d == 0 ? e1y : e3y) + w * ty;
+        const T px = fma(w, tx, fma(u, d == 0 ? e1x : e3x, x0)), py = fma(w, ty, fma(u, d == 0 ? e1y : e3y, y0));
         g = om * mul_sub(px, vy, py, vx);
       }
     } else {
@@ -592,10 +598,10 @@ struct ElemGeo {
 #pragma unroll
       for (int i = 1; i < N; ++i) {
         const T u = cVB<T, N>.Xf[i];
-        const T tx = Ax + u * dx, ty = Ay + u * dy;
+        const T tx = fma(u, dx, Ax), ty = fma(u, dy, Ay);
         vx[i] = sg * ty;
         vy[i] = -sg * tx;
-        const T px = x0 + u * Bx + w * tx, py = y0 + u * By + w * ty;
+        const T px = fma(w, tx, fma(u, Bx, x0)), py = fma(w, ty, fma(u, By, y0));
         vg[i] = om * mul_sub(px, vy[i], py, vx[i]);
       }
     } else {
@@ -619,15 +625,15 @@ struct ElemGeo {
   }
   __device__ __forceinline__ void line_metrics_still(int d, int m, T *vx, T *vy) const {
     if (OTF && tab == nullptr) {
-      // the tangent with the direction's sign, sg (A + u d): a sign commutes
-      // with every rounding
+      // the tangent with the direction's sign, sg (A + u d) in one rounding, as
+      // line_metrics() has it (a sign commutes with it)
       const T sg = d == 0 ? T(1) : T(-1);
       const T Ax = sg * (d == 0 ? e3x : e1x), Ay = sg * (d == 0 ? e3y : e1y), Dx = sg * dx, Dy = sg * dy;
 #pragma unroll
       for (int i = 1; i < N; ++i) {
         const T u = cVB<T, N>.Xf[i];
-        vx[i] = Ay + u * Dy;
-        vy[i] = -(Ax + u * Dx);
+        vx[i] = fma(u, Dy, Ay);
+        vy[i] = -fma(u, Dx, Ax);
       }
     } else {
 #pragma unroll
@@ -649,7 +655,7 @@ struct ElemGeo {
   __device__ __forceinline__ T inv_jac(int i, int j) const {
     if (OTF && tab == nullptr) {
       const T xi = cVB<T, N>.Xs[i], eta = cVB<T, N>.Xs[j];
-      const T xx = e1x + eta * dx, yx = e1y + eta * dy, xe = e3x + xi * dx, ye = e3y + xi * dy;
+      const T xx = fma(eta, dx, e1x), yx = fma(eta, dy, e1y), xe = fma(xi, dx, e3x), ye = fma(xi, dy, e3y);
       return recip(mul_sub(xx, ye, xe, yx));
     }
     return tab[L::iJ + j * N + i];
@@ -667,7 +673,7 @@ struct ElemGeo {
       } else {
         r2 = r[2], r3 = r[3], r4 = r[4], r5 = r[5], r6 = r[6], r7 = r[7];
       }
-      const T xx = r2 + eta * r6, yx = r3 + eta * r7, xe = r4 + xi * r6, ye = r5 + xi * r7;
+      const T xx = fma(eta, r6, r2), yx = fma(eta, r7, r3), xe = fma(xi, r6, r4), ye = fma(xi, r7, r5);
       return recip(mul_sub(xx, ye, xe, yx));
     }
     return ((const T *)md.geo + (size_t)ti * L::G)[L::iJ + j * N + i];
@@ -679,7 +685,7 @@ struct ElemGeo {
     if constexpr (OTF) {
       if (ti < 0) {
         const float4 a = reinterpret_cast<const float4 *>(r)[0], b = reinterpret_cast<const float4 *>(r)[1];
-        const T xx = a.z + eta * b.z, yx = a.w + eta * b.w, xe = b.x + xi * b.z, ye = b.y + xi * b.w;
+        const T xx = fma(eta, b.z, a.z), yx = fma(eta, b.w, a.w), xe = fma(xi, b.z, b.x), ye = fma(xi, b.w, b.y);
         return recip(mul_sub(xx, ye, xe, yx));
       }
     }
@@ -688,7 +694,7 @@ struct ElemGeo {
   // gradients of xi and eta at SP k = j N + i, at (xi, eta) = (X_i, X_j): (xi_x, xi_y), (eta_x, eta_y)
   __device__ __forceinline__ void sp_grad_at(int k, T xi, T eta, T &xix, T &xiy, T &etx, T &ety) const {
     if (OTF && tab == nullptr) {
-      const T xx = e1x + eta * dx, yx = e1y + eta * dy, xe = e3x + xi * dx, ye = e3y + xi * dy;
+      const T xx = fma(eta, dx, e1x), yx = fma(eta, dy, e1y), xe = fma(xi, dx, e3x), ye = fma(xi, dy, e3y);
       const T iJ = T(1) / mul_sub(xx, ye, xe, yx);
       xix = ye * iJ;
       xiy = -xe * iJ;
@@ -712,7 +718,7 @@ struct ElemGeo {
 // pressure from the conservative state with ir = 1 / rho at hand
 template <typename T>
 __device__ __forceinline__ T pressure_ir(const T *q, T ir, T gm1) {
-  return gm1 * fma(-(T(0.5) * mul_add(q[1], q[1], q[2], q[2])), ir, q[3]);
+  return mul_rn(gm1, fma(-(T(0.5) * mul_add(q[1], q[1], q[2], q[2])), ir, q[3]));
 }
 
 template <typename T>
@@ -743,7 +749,7 @@ __device__ __forceinline__ void rusanov(const T *qL, const T *qR, T nx, T ny, T 
   const T gm1 = gamma - T(1);
   const T irL = recip(qL[0]), irR = recip(qR[0]);
   const T pL = pressure_ir(qL, irL, gm1), pR = pressure_ir(qR, irR, gm1);
-  const T unL = mul_add(qL[1], nx, qL[2], ny) * irL, unR = mul_add(qR[1], nx, qR[2], ny) * irR;
+  const T unL = mul_rn(mul_add(qL[1], nx, qL[2], ny), irL), unR = mul_rn(mul_add(qR[1], nx, qR[2], ny), irR);
   const T lL = fabs(unL - vgn) + root(gamma * pL * irL);
   const T lR = fabs(unR - vgn) + root(gamma * pR * irR);
   const T lam = lL > lR ? lL : lR;
@@ -1780,7 +1786,7 @@ struct VolCfg {
 template <typename T>
 __device__ __forceinline__ void point_flux(const T *q, T vx, T vy, T vg, T gm1, T *f) {
   const T ir = recip(q[0]);
-  const T p = gm1 * (q[3] - T(0.5) * mul_add(q[1], q[1], q[2], q[2]) * ir);
+  const T p = pressure_ir(q, ir, gm1);
   const T un = mul_add(q[1], vx, q[2], vy) * ir;
   f[0] = mul_sub(q[0], un, vg, q[0]);
   f[1] = fma(q[1], un, mul_sub(p, vx, vg, q[1]));
@@ -1792,7 +1798,7 @@ __device__ __forceinline__ void point_flux(const T *q, T vx, T vy, T vg, T gm1, 
 template <typename T>
 __device__ __forceinline__ void point_flux_still(const T *q, T vx, T vy, T gm1, T *f) {
   const T ir = recip(q[0]);
-  const T p = gm1 * (q[3] - T(0.5) * mul_add(q[1], q[1], q[2], q[2]) * ir);
+  const T p = pressure_ir(q, ir, gm1);
   const T un = mul_add(q[1], vx, q[2], vy) * ir;
   f[0] = q[0] * un;
   f[1] = fma(q[1], un, p * vx);

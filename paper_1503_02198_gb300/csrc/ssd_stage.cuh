@@ -183,11 +183,12 @@ __device__ __forceinline__ void rusanov2(const float2 *q, const float2 *n, float
   for (int s = 0; s < 2; ++s) {
     const float2 *a = s ? n : q;
     const float2 ir = f2_neg_recip(a[0]);  // -1 / rho
-    const float2 p = f2_mul(ngm1, f2_fma(f2_mul(f2(0.5f), f2_fma(a[1], a[1], f2_mul(a[2], a[2]))), ir, a[3]));  // -p
-    // -V.n (products summed elsewhere are formed by an FMA with 0: the compiler
+    // (products summed elsewhere are formed by an FMA with 0: the compiler
     // fuses a plain multiply with a later sum, which rounds otherwise)
+    const float2 e = f2_fma(f2_mul(f2(0.5f), f2_fma(a[1], a[1], f2_mul(a[2], a[2]))), ir, a[3]);
+    const float2 p = f2_fma(ngm1, e, f2(0.0f));  // -p
     const float2 mn = f2_fma(a[1], nx, f2_mul(a[2], ny));
-    const float2 un = MOVING ? f2_mul(mn, ir) : f2_fma(mn, ir, f2(0.0f));
+    const float2 un = f2_fma(mn, ir, f2(0.0f));  // -V.n
     const float2 h = f2_sub(a[3], p);
     if (MOVING) {
       f[s][0] = f2_fma(a[0], un, f2_mul(vg, a[0]));
@@ -477,7 +478,7 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
     // fluxes at its interior points, its part of the divergence ----
     {
       // a cell of the stationary zone: no rotation, no grid velocity (the same
-      // bits as with the identity and zero)
+      // bits as with the identity and zero, every sum's rounding being written out)
       const bool moving = (sEF[le] & kZoneMask) != 0;
       ElemGeo<float, N, true> Gm;
       if (moving) Gm.load_rec(md, e0 + le, sEF[le], sEG + le * 8, sZT);

@@ -1,0 +1,43 @@
+"""Roundings of the kernels that no tolerance of the parity tests sees."""
+import numpy as np
+import pytest
+
+from ssd_inputs import fields, meshes
+from ssd_inputs.workloads import FlowParams
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ssd():
+    import paper_1503_02198_gb300 as pkg
+    pkg.build()
+    return pkg
+
+
+def _skewed(zone, cubic=False):
+    """A channel of cells that are no parallelograms, all in one zone."""
+    return meshes.channel_mesh(17, 11, 3.0, 2.0, cubic=cubic, zone=zone,
+                               mapping=lambda x, y: (x + 0.07 * x * y, y + 0.05 * x * y + 0.03 * x))
+
+
+@pytest.mark.parametrize("N", [3, 4, 5, 6])
+@pytest.mark.parametrize("precision", [1, 2])
+@pytest.mark.parametrize("cubic", [False, True])
+def test_stationary_cells_round_as_the_general_form(ssd, precision, N, cubic):
+    """FP32 Euler: the branch for cells without rotation and grid velocity against
+    the general one on a zone at rest at angle 0.  Every sum rounds the same way in
+    both, so residuals and states are equal bit for bit."""
+    R, S = [], []
+    for zone in (0, 1):
+        for rk in (3, 5):
+            s = ssd.Solver(_skewed(zone, cubic), N - 1, FlowParams(omega=0.0, u_inf=0.3, rk_stages=rk), precision=precision)
+            Q = s.state_from(lambda x, y: fields.random_smooth_state(x, y, seed=N, amp=0.05, scale=3.0))
+            s.sd_set_state(Q)
+            R.append(s.sd_residual())
+            s.sd_step(2e-4, 10)
+            s.sd_sync()
+            S.append(s.sd_get_state())
+            s.close()
+    assert np.array_equal(R[0], R[2]) and np.array_equal(R[1], R[3])
+    assert np.array_equal(S[0], S[2]) and np.array_equal(S[1], S[3])
