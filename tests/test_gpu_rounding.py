@@ -15,6 +15,26 @@ def ssd():
     return pkg
 
 
+def _rest_with_density_jumps(ssd, oracle_mod, precision, zone, N, E0):
+    """Relative L2 error of the density residual of fluid at rest with total energy E0
+    and a density of its own in every cell: only the Rusanov jump term, half the
+    sound speed times the jump, is left."""
+    SLIP = meshes.BC_SLIP
+    m = meshes.channel_mesh(9, 7, 3.0, 2.0, tags=(SLIP,) * 4, zone=zone)
+    prm = FlowParams(omega=0.0)
+    E = len(m["elem_nodes"])
+    Q = np.zeros((E, 4, N, N))
+    Q[:, 0] = np.random.Generator(np.random.PCG64(N)).uniform(0.5, 1.5, E)[:, None, None]
+    Q[:, 3] = E0
+    s = ssd.Solver(m, N - 1, prm, precision=precision)
+    s.sd_set_state(Q)
+    R = s.sd_residual()[:, 0]
+    s.close()
+    ref = oracle_mod.Oracle(m, N, prm).residual(Q, 0.0)[:, 0]
+    scale = np.abs(ref).max()
+    return float(np.sqrt(((R / scale - ref / scale) ** 2).sum() / ((ref / scale) ** 2).sum()))
+
+
 def _skewed(zone, cubic=False):
     """A channel of cells that are no parallelograms, all in one zone."""
     return meshes.channel_mesh(17, 11, 3.0, 2.0, cubic=cubic, zone=zone,
@@ -41,3 +61,14 @@ def test_stationary_cells_round_as_the_general_form(ssd, precision, N, cubic):
             s.close()
     assert np.array_equal(R[0], R[2]) and np.array_equal(R[1], R[3])
     assert np.array_equal(S[0], S[2]) and np.array_equal(S[1], S[3])
+
+
+@pytest.mark.parametrize("N", [3, 4, 5, 6])
+@pytest.mark.parametrize("precision", [1, 2])
+@pytest.mark.parametrize("zone", [0, 1])
+def test_fp32_sound_speed_of_a_subnormal_square(ssd, oracle_mod, precision, zone, N):
+    """gamma p / rho = 5.6e-41, a subnormal float with spacing 1.4e-45 (2.5e-5 of it):
+    N roundings of the trace of E, three of p and of the square, each half a
+    spacing of values down to 4e-41 (1.8e-5), halved by the root: (N + 3) 0.9e-5
+    <= 8.1e-5; twice that is allowed."""
+    assert _rest_with_density_jumps(ssd, oracle_mod, precision, zone, N, 1e-40) <= 1.7e-4
