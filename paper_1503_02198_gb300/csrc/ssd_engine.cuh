@@ -231,26 +231,6 @@ __device__ __forceinline__ T recip(T x) {
   return recip_newton(x);
 }
 
-// Square root: the hardware's in FP32; in FP64 Goldschmidt's iteration (a
-// coupled Newton iteration for sqrt(x) and 1 / (2 sqrt(x))) from the hardware's
-// approximate reciprocal root, two steps and a last residual correction, ten
-// FP64 instructions, within an ulp or so; 0 for 0, NaN for negative x.
-__device__ __forceinline__ float root(float x) { return sqrtf(x); }
-__device__ __forceinline__ double root(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double g = x * y, h = 0.5 * y;
-  double r = fma(-g, h, 0.5);
-  g = fma(g, r, g);
-  h = fma(h, r, h);
-  r = fma(-g, h, 0.5);
-  g = fma(g, r, g);
-  h = fma(h, r, h);
-  g = fma(fma(-g, g, x), h, g);
-  // (x = 0: the reciprocal root is infinite)
-  return (__double2hiint(x) | __double2loint(x)) == 0 ? 0.0 : g;
-}
-
 // face f of an element: sign sigma_f with F~_end = sigma_f |S| F.n_out
 __device__ __forceinline__ double face_sigma(int f) { return (f == 1 || f == 2) ? 1.0 : -1.0; }
 
@@ -743,15 +723,18 @@ __device__ __forceinline__ void normal_flux(const T *q, T p, T nx, T ny, T vgn, 
 }
 
 // Rusanov common flux (Sec. 3.1) for unit normal n from L to R; one
-// reciprocal density per side
+// reciprocal density per side.  The sound speeds are CUDA's sqrt: in FP64
+// Goldschmidt's iteration from the approximate reciprocal root was within an ulp
+// and no faster (a step of 246,900 cells at N = 6: 9505 us, with sqrt 9450), and
+// gave NaN where the square is subnormal.
 template <typename T>
 __device__ __forceinline__ void rusanov(const T *qL, const T *qR, T nx, T ny, T vgn, T gamma, T *Fn) {
   const T gm1 = gamma - T(1);
   const T irL = recip(qL[0]), irR = recip(qR[0]);
   const T pL = pressure_ir(qL, irL, gm1), pR = pressure_ir(qR, irR, gm1);
   const T unL = mul_rn(mul_add(qL[1], nx, qL[2], ny), irL), unR = mul_rn(mul_add(qR[1], nx, qR[2], ny), irR);
-  const T lL = fabs(unL - vgn) + root(gamma * pL * irL);
-  const T lR = fabs(unR - vgn) + root(gamma * pR * irR);
+  const T lL = fabs(unL - vgn) + sqrt(gamma * pL * irL);
+  const T lR = fabs(unR - vgn) + sqrt(gamma * pR * irR);
   const T lam = lL > lR ? lL : lR;
   if constexpr (std::is_same<T, double>::value) {
     // the FP64 pipe's way: both sides' fluxes as one sum, the grid velocity

@@ -72,3 +72,10 @@ def test_fp32_sound_speed_of_a_subnormal_square(ssd, oracle_mod, precision, zone
     spacing of values down to 4e-41 (1.8e-5), halved by the root: (N + 3) 0.9e-5
     <= 8.1e-5; twice that is allowed."""
     assert _rest_with_density_jumps(ssd, oracle_mod, precision, zone, N, 1e-40) <= 1.7e-4
+
+
+@pytest.mark.parametrize("N", [3, 4, 5, 6])
+def test_fp64_sound_speed_of_a_subnormal_square(ssd, oracle_mod, N):
+    """The same in FP64, E = 1e-310: spacing 4.9e-324, so (N + 3) times
+    4.9e-324 / 4e-311 / 4 = 3.1e-14, twice that on each of the two sides compared."""
+    assert _rest_with_density_jumps(ssd, oracle_mod, 0, 0, N, 1e-310) <= 1.2e-12
