@@ -2,6 +2,7 @@
 import numpy as np
 import pytest
 
+from helpers import small_rotor, small_twin
 from ssd_inputs import fields, meshes
 from ssd_inputs.workloads import FlowParams
 
@@ -79,3 +80,39 @@ def test_fp64_sound_speed_of_a_subnormal_square(ssd, oracle_mod, N):
     """The same in FP64, E = 1e-310: spacing 4.9e-324, so (N + 3) times
     4.9e-324 / 4e-311 / 4 = 3.1e-14, twice that on each of the two sides compared."""
     assert _rest_with_density_jumps(ssd, oracle_mod, 0, 0, N, 1e-310) <= 1.2e-12
+
+
+# relative L2 error of the FP64 residual against the extended oracle with every
+# contraction a plain chain of FMAs over the weights and the two sides' fluxes
+# formed apart, by mesh and N (the cases of _fp64_residual_error)
+PLAIN = {("rotor", 3): 2.769e-14, ("rotor", 4): 2.071e-14, ("rotor", 5): 2.743e-14, ("rotor", 6): 2.683e-14,
+         ("twin", 3): 1.421e-14, ("twin", 4): 1.01e-14, ("twin", 5): 1.193e-14, ("twin", 6): 1.32e-14}
+
+
+def _fp64_residual_error(ssd, oracle_mod, kind, N):
+    """Root mean square over four smooth states."""
+    mesh, prm = (small_rotor(scale=2, shift_R=0.05), FlowParams(omega=0.8)) if kind == "rotor" else \
+        (small_twin(n_core2=5), FlowParams(omega=0.6))
+    ext = oracle_mod.Oracle(mesh, N, prm, real="long")
+    s = ssd.Solver(mesh, N - 1, prm, precision=0)
+    e2 = []
+    for seed in range(4):
+        t = 0.3 + 0.7 * seed
+        Q = s.state_from(lambda x, y: fields.random_smooth_state(x, y, seed=10 * N + seed, amp=0.2, scale=3.0))
+        s.sd_set_state(Q)
+        s.sd_set_time(t)
+        ref = ext.residual(Q, t)
+        d = s.sd_residual().astype(np.longdouble) - ref
+        e2.append(float((d ** 2).sum() / (ref ** 2).sum()))
+    s.close()
+    return float(np.sqrt(np.mean(e2)))
+
+
+@pytest.mark.parametrize("N", [3, 4, 5, 6])
+@pytest.mark.parametrize("kind", ["rotor", "twin"])
+def test_fp64_residual_error_no_larger_than_the_plain_form(ssd, oracle_mod, kind, N):
+    """Folded sums and joint fluxes may not round worse than the plain form.  The
+    error is a mean over 1e5 values and more, so 1 % is beyond its scatter."""
+    e = _fp64_residual_error(ssd, oracle_mod, kind, N)
+    print(f"{kind} N={N}: {e:.4g}, plain {PLAIN[kind, N]:.4g}")
+    assert e <= 1.01 * PLAIN[kind, N]
