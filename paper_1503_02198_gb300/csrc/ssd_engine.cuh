@@ -631,15 +631,6 @@ struct ElemGeo {
     else if (f == 0) eta_fp(j, 0, vx, vy, g);
     else eta_fp(j, N, vx, vy, g);
   }
-  // 1 / |J| at SP (X_i, X_j)
-  __device__ __forceinline__ T inv_jac(int i, int j) const {
-    if (OTF && tab == nullptr) {
-      const T xi = cVB<T, N>.Xs[i], eta = cVB<T, N>.Xs[j];
-      const T xx = fma(eta, dx, e1x), yx = fma(eta, dy, e1y), xe = fma(xi, dx, e3x), ye = fma(xi, dy, e3y);
-      return recip(mul_sub(xx, ye, xe, yx));
-    }
-    return tab[L::iJ + j * N + i];
-  }
   // 1 / |J| at SP (X_i, X_j) straight from the cell flag and the unrotated
   // record or table (|J| does not change under the rotation)
   static __device__ __forceinline__ T inv_jac_t0(const MeshDev &md, int f, const T *r, int i, int j) {
@@ -3008,20 +2999,6 @@ struct EngineImpl : Engine {
   }
   StatePtr C() const override { return StatePtr{sC[0], sC[1]}; }
   void *W() const override { return sW; }
-
-  // launch shapes chosen by the batch autotuner: volume CTAs per SM (capped
-  // by occupancy; 0 keeps the current value) and the face-kernel block size
-  void tuning(int *vol_ctas_per_sm, int *max_ctas_per_sm, int *fblock) override {
-    if (max_ctas_per_sm) *max_ctas_per_sm = occ_rk;
-    if (vol_ctas_per_sm) {
-      if (*vol_ctas_per_sm > 0) grid_rk = std::min(*vol_ctas_per_sm, occ_rk) * sms;
-      *vol_ctas_per_sm = grid_rk / sms;
-    }
-    if (fblock) {
-      if (*fblock > 0) face_block = std::min(*fblock, face_block_max);
-      *fblock = face_block;
-    }
-  }
 
   void advance(const MeshDev &md, double dt, cudaStream_t s) override {
     launch_pdl(k_advance, 1, 1, 0, s, md.clk, dt);

@@ -237,8 +237,6 @@ struct Engine {
   // the number of its tiles without an interface or boundary face (they come
   // first in md.tord)
   virtual void set_early_tiles(int n) = 0;
-  // get / set the tunable launch shapes (see EngineImpl::tuning)
-  virtual void tuning(int *vol_ctas_per_sm, int *max_ctas_per_sm, int *face_block) = 0;
   // the two state buffers A and B: E elements, storage for Epad >= E
   virtual cudaError_t alloc_state(int E, int Epad) = 0;
   virtual StatePtr A() const = 0;

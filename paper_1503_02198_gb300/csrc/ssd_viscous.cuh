@@ -215,8 +215,6 @@ struct VisCfg {
   static constexpr bool F = sizeof(T) == 4;
   static constexpr int EPB = N == 3 ? 16 : (N == 4 ? 8 : (N == 5 ? (F ? 4 : 8) : (F ? 8 : 4)));
   static constexpr int THREADS = EPB * 2 * N;
-  // resident blocks per SM the register budget is set for: about 16 warps
-  static constexpr int MINB = 16 / ((THREADS + 31) / 32) > 0 ? 16 / ((THREADS + 31) / 32) : 1;
 };
 
 // Gradients at the SPs of a tile (thread per SP line, then per SP): on
