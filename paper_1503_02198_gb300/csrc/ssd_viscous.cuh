@@ -517,12 +517,15 @@ struct VisVolCfg {
   static_assert(QE % 16 == 0 && GE % 16 == 0 && CE % 16 == 0, "bulk-copy sizes and alignment");
   static_assert(SMEM <= 227 * 1024 && THREADS <= 1024, "one CTA");
   // resident CTAs per SM the register budget is set for (warps per SM), or what
-  // the shared memory admits.  us a step for 16 / 20 / 25 / 32 warps: FP32 N = 3
-  // (288 cells) 55.7 / 55.8 / 56.4 / 60.0, N = 4 (14,752 cells, five stages)
-  // 176 / 168 / 160 / 161, N = 5 (20,096 cells) 179 / 168 / 173 / 176; FP64 N = 5
-  // 1856 / 1865 / 1865 / 1866
+  // the shared memory admits.  us for 16 / 20 / 25 / 32 warps, FP32, three steps of
+  // the 20,096-cell ellipse: N = 3 304 / 285 / 282 / 283, N = 4 358 / 352 / 344 / 336,
+  // N = 5 546 / 518 / 518 / 550, N = 6 767 / 767 / 708 / 745; of a 10,368-cell
+  // Couette gap N = 3 241 / 229 / 236 / 236, N = 6 474 / 474 / 448 / 484; two
+  // five-stage steps of the 14,752-cell tank at N = 4 352 / 336 / 320 / 322; 288
+  // cells at N = 3, one step 55.7 / 55.8 / 56.4 / 60.0.  FP64, one step of the
+  // ellipse: within 0.6 % of each other at every N.
   static constexpr int WARPS = (THREADS + 31) / 32;
-  static constexpr int BUDGET = sizeof(T) == 4 ? (N == 4 ? 25 : 20) : 16;
+  static constexpr int BUDGET = sizeof(T) == 4 ? (N == 4 || N == 6 ? 25 : 20) : 16;
   static constexpr int BY_WARPS = BUDGET / WARPS > 0 ? BUDGET / WARPS : 1;
   static constexpr int BY_SMEM = 228 * 1024 / (SMEM + 1024);
   static constexpr int MINB = BY_WARPS < BY_SMEM ? BY_WARPS : (BY_SMEM > 0 ? BY_SMEM : 1);
