@@ -117,13 +117,13 @@ struct VolBasis {
   T Dm[N * (N + 1)];  // l'_{i+1/2}(X_k) [k][i]
   T H0[N], H1[N];     // h_k(0), h_k(1)
   T Xs[N], Xf[N + 1]; // solution and flux points
-  // Even and odd halves of the weights (FP64 path): the points are symmetric, so
-  // with sums and differences of mirrored values each half needs half of the
-  // multiplications.  Interpolation to FPs i and N - i: half (h_k +- h_{N-1-k}) at
-  // X_{i+1/2}, i = 1 .. N/2; derivative at SPs k and N - 1 - k: half (l'_i +- l'_{N-i})
-  // at X_k; for the middle point of an odd number the weight itself.
-  T He[(N / 2 + 1) * ((N + 1) / 2)], Ho[(N / 2 + 1) * ((N + 1) / 2)];
-  T De[((N + 1) / 2) * (N / 2 + 1)], Do[((N + 1) / 2) * (N / 2 + 1)];
+  // Even and odd halves of the weights (FP64 path, N = 6): the points are
+  // symmetric, so with sums and differences of mirrored values each half needs
+  // half of the multiplications.  Interpolation to FPs i and N - i: half
+  // (h_k +- h_{N-1-k}) at X_{i+1/2}, i = 1 .. N/2; derivative at SPs k and
+  // N - 1 - k: half (l'_i +- l'_{N-i}) at X_k, for the middle FP the weight itself.
+  T He[(N / 2 + 1) * (N / 2)], Ho[(N / 2 + 1) * (N / 2)];
+  T De[(N / 2) * (N / 2 + 1)], Do[(N / 2) * (N / 2 + 1)];
   // the same weights duplicated into float pairs for packed FP32x2 FMAs
   float2 Hf2[(N + 1) * N], Dm2[N * (N + 1)], H02[N], H12[N];
 };
@@ -2194,11 +2194,14 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
             sRG[le][(3) * NN + sp] = acc2[1][k].y;
           }
         }
-      } else if constexpr (N <= 4) {
-        // FP64, bound by the FP64 pipe.  Up to N = 4 sums and differences of
-        // mirrored values (below) save at most two of 32 instructions per line and
-        // variable and round worse (N = 4: 1.14 to 1.19 times the residual's error):
-        // weights as they are.
+      } else if constexpr (N <= 5) {
+        // FP64, bound by the FP64 pipe.  Up to N = 5 the weights as they are: with
+        // sums and differences of mirrored values (below) N = 4 saves two of 32
+        // instructions per line and variable and the residual's error is 1.14 to
+        // 1.19 times as large; N = 5 saves four of 50 (the residual of 6,016 cells
+        // 56.7 us instead of 58.7) and is nearer to the extended oracle (0.96 to
+        // 0.98) but further from the same method in plain 64 bits (1.06), which
+        // shares the rounded weights of this form.
         T q[4][N], acc[4][N];
 #pragma unroll
         for (int k = 0; k < N; ++k)
@@ -2236,18 +2239,19 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
 #pragma unroll
           for (int v = 0; v < 4; ++v) o[v * NN + (d == 0 ? mline * N + k : k * N + mline)] = acc[v][k];
       } else {
-        // FP64, N = 5 and 6.  Values at mirrored points are taken as sums and
-        // differences (VolBasis).  The derivative is that of the fluxes less the
-        // one at the line's start, r (a constant has none): the sums of mirrored
-        // fluxes would else be rounded at twice a flux's size.  The residual's error
-        // is 0.83 to 0.98 times the plain form's (without r 1.00 to 1.07).  At N = 6
-        // the interpolation of a line takes 25 instructions per variable instead of
-        // 30, its derivative 37 instead of 42; a step of 246,900 cells takes 9815 us
-        // (9450 without r; 11335 plain and without the form for cells at rest).  A
-        // pair of FPs (i, N - i) at a time: interpolation, fluxes, and their part of
-        // the divergence; on cells of the stationary zone without rotation and grid
+        // FP64, N = 6.  Values at mirrored points are taken as sums and differences
+        // (VolBasis).  The derivative is that of the fluxes less the one at the
+        // line's start, r (a constant has none): the sums of mirrored fluxes would
+        // else be rounded at twice a flux's size.  The residual's error is 0.83 to
+        // 0.88 times the plain form's (without r 1.03 to 1.07).  The interpolation
+        // of a line takes 25 instructions per variable instead of 30, its derivative
+        // 37 instead of 42; a step of 246,900 cells takes 9790 us (9450 without r;
+        // 11335 plain and without the form for cells at rest).  A pair of FPs
+        // (i, N - i) at a time: interpolation, fluxes, and their part of the
+        // divergence; on cells of the stationary zone without rotation and grid
         // velocity.
-        constexpr int HK = (N + 1) / 2, HI = N / 2 + 1;
+        constexpr int HK = N / 2, HI = N / 2 + 1;
+        static_assert(N % 2 == 0, "no SP mirrors itself");
         T qe[4][HK], qo[4][HK];
 #pragma unroll
         for (int k = 0; k < HK; ++k)
@@ -2255,13 +2259,9 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
           for (int v = 0; v < 4; ++v) {
             const int k2 = N - 1 - k;
             const T x = d == 0 ? sQ[le][v * NN + mline * N + k] : sQ[le][v * NN + k * N + mline];
-            if (k2 == k) {
-              qe[v][k] = x;
-            } else {
-              const T y = d == 0 ? sQ[le][v * NN + mline * N + k2] : sQ[le][v * NN + k2 * N + mline];
-              qe[v][k] = x + y;
-              qo[v][k] = x - y;
-            }
+            const T y = d == 0 ? sQ[le][v * NN + mline * N + k2] : sQ[le][v * NN + k2 * N + mline];
+            qe[v][k] = x + y;
+            qo[v][k] = x - y;
           }
         T X[4][HK], Y[4][HK];  // divergence at SPs k and N - 1 - k: Y + X and Y - X
         T r[4];
@@ -2289,7 +2289,7 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
               } else {
                 T o = qo[v][0] * B.Ho[i * HK];
 #pragma unroll
-                for (int k = 1; k < N / 2; ++k) o = fma(qo[v][k], B.Ho[i * HK + k], o);
+                for (int k = 1; k < HK; ++k) o = fma(qo[v][k], B.Ho[i * HK + k], o);
                 sa[v] = e + o;
                 sb2[v] = e - o;
               }
@@ -2312,8 +2312,7 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
           for (int k = 0; k < HK; ++k)
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-              if (2 * k != N - 1)
-                X[v][k] = i == 0 ? B.De[k * HI] * fe[v] : fma(B.De[k * HI + i], fe[v], X[v][k]);
+              X[v][k] = i == 0 ? B.De[k * HI] * fe[v] : fma(B.De[k * HI + i], fe[v], X[v][k]);
               if (i2 != i) Y[v][k] = i == 0 ? B.Do[k * HI] * fo[v] : fma(B.Do[k * HI + i], fo[v], Y[v][k]);
             }
         }
@@ -2323,14 +2322,8 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
             const int k2 = N - 1 - k;
-            const int p1 = v * NN + (d == 0 ? mline * N + k : k * N + mline);
-            const int p2 = v * NN + (d == 0 ? mline * N + k2 : k2 * N + mline);
-            if (k2 == k) {
-              o[p1] = Y[v][k];
-            } else {
-              o[p1] = Y[v][k] + X[v][k];
-              o[p2] = Y[v][k] - X[v][k];
-            }
+            o[v * NN + (d == 0 ? mline * N + k : k * N + mline)] = Y[v][k] + X[v][k];
+            o[v * NN + (d == 0 ? mline * N + k2 : k2 * N + mline)] = Y[v][k] - X[v][k];
           }
       }
     }
@@ -2700,13 +2693,12 @@ struct EngineImpl : Engine {
     }
     for (int k = 0; k <= N; ++k) vb.Xf[k] = (T)hb.Xf[k];
     for (int i = 0; i <= N / 2; ++i)
-      for (int k = 0; k < (N + 1) / 2; ++k) {
-        const bool mid = 2 * k == N - 1;  // the SP that mirrors itself
+      for (int k = 0; k < N / 2; ++k) {
         const double a = hb.Hf[i * N + k], b = hb.Hf[i * N + N - 1 - k];
-        vb.He[i * ((N + 1) / 2) + k] = (T)(mid ? a : 0.5 * (a + b));
-        vb.Ho[i * ((N + 1) / 2) + k] = (T)(mid ? 0.0 : 0.5 * (a - b));
+        vb.He[i * (N / 2) + k] = (T)(0.5 * (a + b));
+        vb.Ho[i * (N / 2) + k] = (T)(0.5 * (a - b));
       }
-    for (int k = 0; k < (N + 1) / 2; ++k)
+    for (int k = 0; k < N / 2; ++k)
       for (int i = 0; i <= N / 2; ++i) {
         const bool mid = 2 * i == N;  // the FP that mirrors itself
         const double a = hb.Dm[k * (N + 1) + i], b = hb.Dm[k * (N + 1) + N - i];
