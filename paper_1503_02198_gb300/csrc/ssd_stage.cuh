@@ -18,11 +18,12 @@
 // one trace buffer (TR) and writes another (TRo).
 //
 // What bounds it (N = 6, 246,900 cells, double-float state): shared-memory
-// bandwidth 69 %, issue 49 %, DRAM 1.03 GB per later stage (4.9 TB/s); barrier,
-// wait and shared-load stalls 1.3 each per issue with 15 warps per SM.  A step
-// took 703 us with the face pass (48 us) and the volume kernel (180 us) apart
-// and takes 598 us here (float state, 123,450 cells: 322 -> 282 us; 31,509 cells
-// at N = 3: 72 -> 53 us; 6,016 cells at N = 4: 39 -> 29 us).
+// bandwidth 69 %, issue 50 %, DRAM 1.03 GB in the 207 us of a later stage (5.0
+// TB/s); barrier, wait and shared-load stalls 1.2 to 1.3 each per issue with 15
+// warps per SM.  A step took 703 us with the face pass (48 us) and the volume
+// kernel (180 us) apart and takes 606 us here (float state, 123,450 cells: 322 ->
+// 286 us; 31,509 cells at N = 3: 72 -> 53 us; 6,016 cells at N = 4: 39 -> 29 us).
+// Results are the bits of the separate kernels.
 #pragma once
 
 namespace ssd {
@@ -236,9 +237,13 @@ struct StageCfg {
   static constexpr int TXA = EPB * QE + EGB + EFB;
   static_assert((SE * 4) % 16 == 0 && QE % 16 == 0 && QB % 16 == 0 && RECB % 16 == 0 && O_QLO % 16 == 0, "bulk copies");
   static constexpr int BY_SMEM = 228 * 1024 / (SMEM + 1024);
-  // 15 to 20 warps per SM with 128 registers: a sixth CTA needs a cap of 96, and
-  // the few words that spill then come back from L2 (the tiles take the L1):
-  // 836 us a step instead of 656 on 246,900 cells at N = 6
+  // five CTAs of three warps (N = 3, 4 and 6) have 128 registers a thread.  A sixth
+  // needs a cap of 96, and the words that spill then come back from L2 (the tiles
+  // take the L1): 836 us a step instead of 656 on 246,900 cells at N = 6.  At N = 5
+  // a CTA has four warps: shared memory admits four with a double-float state (128
+  // registers); with a float state five fit at 96 registers, and there five are
+  // better although the residual's form spills two words (three steps of 96,256
+  // cells 616 us, 665 with four; 24,064 cells 208 and 218; 6,016 cells 112 and 106)
   static constexpr int MINB = BY_SMEM < 5 ? BY_SMEM : 5;
 };
 
@@ -349,8 +354,8 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
   int item = blockIdx.x;
   // item i's tile; rev: the early tiles from the last to the first, so that a
   // stage begins on what the stage before it wrote last, still in L2 (the trace
-  // buffers alternate, and with them the direction): 604 -> 598 us a step on
-  // 246,900 cells, 284 -> 282 on 123,450 with float state
+  // buffers alternate, and with them the direction): 1 % of a step on 246,900
+  // cells, 0.7 % on 123,450 with float state
   auto tile_of = [&](int i) { return i < nitems ? md.tord[rev && i < nearly ? nearly - 1 - i : i] : -1; };
   int tile = tile_of(item), tile1 = tile_of(item + G), tile2 = tile_of(item + 2 * G);
   __syncthreads();
