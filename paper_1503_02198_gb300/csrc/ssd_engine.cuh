@@ -631,26 +631,10 @@ struct ElemGeo {
     else if (f == 0) eta_fp(j, 0, vx, vy, g);
     else eta_fp(j, N, vx, vy, g);
   }
-  // 1 / |J| at SP (X_i, X_j) straight from the cell flag and the unrotated
-  // record or table (|J| does not change under the rotation)
-  static __device__ __forceinline__ T inv_jac_t0(const MeshDev &md, int f, const T *r, int i, int j) {
-    const int ti = ((f & ~kIfaceBit) >> kZoneBits) - 1;
-    if (OTF && ti < 0) {
-      const T xi = cVB<T, N>.Xs[i], eta = cVB<T, N>.Xs[j];
-      T r2, r3, r4, r5, r6, r7;
-      if constexpr (std::is_same<T, float>::value) {
-        const float4 a = reinterpret_cast<const float4 *>(r)[0], b = reinterpret_cast<const float4 *>(r)[1];
-        r2 = a.z, r3 = a.w, r4 = b.x, r5 = b.y, r6 = b.z, r7 = b.w;
-      } else {
-        r2 = r[2], r3 = r[3], r4 = r[4], r5 = r[5], r6 = r[6], r7 = r[7];
-      }
-      const T xx = fma(eta, r6, r2), yx = fma(eta, r7, r3), xe = fma(xi, r6, r4), ye = fma(xi, r7, r5);
-      return recip(mul_sub(xx, ye, xe, yx));
-    }
-    return ((const T *)md.geo + (size_t)ti * L::G)[L::iJ + j * N + i];
-  }
-  // the same at SP sp = j N + i with its coordinates (X_i, X_j) at hand: a warp's
-  // threads take different SPs, and constant memory serves one address at a time
+  // 1 / |J| at SP sp = j N + i, straight from the cell flag and the unrotated
+  // record or table (|J| does not change under the rotation), with the SP's
+  // coordinates xi = X_i, eta = X_j at hand: a warp's threads take different SPs,
+  // and constant memory serves one address at a time
   static __device__ __forceinline__ T inv_jac_at(const MeshDev &md, int f, const T *r, int sp, T xi, T eta) {
     const int ti = ((f & ~kIfaceBit) >> kZoneBits) - 1;
     if constexpr (OTF) {
@@ -2342,7 +2326,7 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
     // ---- phase 2: dQ/dt at the SPs and the Runge-Kutta combination ----
     for (int idx = threadIdx.x; idx < ne * NN; idx += NT) {
       const int l2 = idx / NN, sp = idx - l2 * NN;
-      const T iJ = ElemGeo<T, N, OTF>::inv_jac_t0(md, sEF[l2], sEG + l2 * 8, sp % N, sp / N);
+      const T iJ = ElemGeo<T, N, OTF>::inv_jac_at(md, sEF[l2], sEG + l2 * 8, sp, B.Xs[sp % N], B.Xs[sp / N]);
       const size_t gi = ((size_t)(e0 + l2) * 4) * NN + sp;
       if (MODE == MODE_RESIDUAL) {
 #pragma unroll
