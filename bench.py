@@ -103,7 +103,7 @@ class ClockSampler:
 # header up to the viscous path, and ssd_stage.cuh); otherwise null.
 PROFILED_TRAFFIC = {
     "bytes": 933.3e6,
-    "kernel_sha256": "bbcf5da951c314b9cd57722a7d0aac34b395d13cf11ca9c2a5f2044ca7779dba"}
+    "kernel_sha256": "53ee11f43ccb110c4c7cce2f12869cbae1b2851cec2b589681ba838b4db29039"}
 
 
 def volume_kernel_source():

@@ -1672,6 +1672,16 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
                : "memory");
 }
 
+// The first tile of CTA 0 under the test switch of sd_test_wait_timeout: its wait
+// gives up after a few polls, on a barrier armed with more bytes than the tile's
+// copies deliver, so they may still be in flight.  Delivers the missing bytes (the
+// tile's first cell flags once more, at ef) and waits with the full limit.
+__device__ __forceinline__ void settle_test_wait(const MeshDev &md, void *ef, int e0, uint64_t *bar) {
+  if (md.test_tx_extra == 0) return;
+  bulk_g2s(ef, md.eflag + e0, md.test_tx_extra, bar);
+  mbar_wait_bounded(bar, 0);
+}
+
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -2072,6 +2082,7 @@ __global__ void __launch_bounds__(VolCfg<T, N, OTF, AUX, LO, EPBX, TC>::THREADS,
       if (threadIdx.x == 0) {
         atomicOr(&md.clk->flags, 4);
         // let the copies in flight land before the CTA exits (full limits)
+        if (item == 0) settle_test_wait(md, smem + C::O_EF, tile * EPB, &bar[0]);
         if (next < nitems) mbar_wait_bounded(&bar[st ^ 1], (uint32_t)(((it + 1) >> 1) & 1));
         if (txB) mbar_wait_bounded(&bar[2], (uint32_t)(it & 1));
       }

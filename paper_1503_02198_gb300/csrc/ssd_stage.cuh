@@ -419,11 +419,10 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
 
   // gives up on this CTA: reports the timeout and lets the copies in flight
   // land (full limits) before the CTA exits
-  auto give_up = [&](int it, bool a_pending, bool b_issued) {
+  auto give_up = [&](int it, bool b_issued) {
     asm volatile("cp.async.wait_all;" ::: "memory");
     if (threadIdx.x != 0) return;
     atomicOr(&md.clk->flags, 4);
-    if (a_pending) mbar_wait_bounded(&bar[it & 1], (uint32_t)((it >> 1) & 1));
     if (tile1 >= 0) mbar_wait_bounded(&bar[(it + 1) & 1], (uint32_t)(((it + 1) >> 1) & 1));
     if (b_issued) mbar_wait_bounded(&bar[2], (uint32_t)(it & 1));
   };
@@ -455,7 +454,8 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
     }
     if (!cta_wait(&bar[st], (uint32_t)((it >> 1) & 1),
                   (blockIdx.x == 0 && it == 0 && md.test_poll) ? md.test_poll : kWaitPolls)) {
-      give_up(it, false, txB != 0);
+      if (threadIdx.x == 0 && blockIdx.x == 0 && it == 0) settle_test_wait(md, smem + C::O_EF, tile * EPB, &bar[0]);
+      give_up(it, txB != 0);
       return;
     }
     unsigned char *sb = smem + st * C::STAGE;
@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
           bool done = true;
           if (threadIdx.x == 0) done = wait_coupling(&md.clk->done, nblk);
           if (!__syncthreads_and(done)) {
-            give_up(it, false, txB != 0);
+            give_up(it, txB != 0);
             return;
           }
           ready = true;
@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(StageCfg<N, AUX, LO>::THREADS, StageCfg<N, AUX
     // the Runge-Kutta inputs must have landed too
     if (txB) {
       if (!cta_wait(&bar[2], (uint32_t)(it & 1))) {
-        give_up(it, false, false);
+        give_up(it, false);
         return;
       }
     } else {
