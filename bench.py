@@ -103,7 +103,7 @@ class ClockSampler:
 # header up to the viscous path, and ssd_stage.cuh); otherwise null.
 PROFILED_TRAFFIC = {
     "bytes": 933.3e6,
-    "kernel_sha256": "53ee11f43ccb110c4c7cce2f12869cbae1b2851cec2b589681ba838b4db29039"}
+    "kernel_sha256": "c5788888eef132124464ec7296df5e2ae9739ef6e55be9b1bc087123f31ecb1d"}
 
 
 def volume_kernel_source():

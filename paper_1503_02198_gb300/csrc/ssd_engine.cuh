@@ -167,10 +167,6 @@ struct GeoLayout {
 // from the general form.  Such sums are an explicit fma() below, and a product
 // that is used both in a sum and elsewhere (the pressure) is rounded once by
 // mul_rn().
-// a product that is never fused into a later addition
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-
 template <typename T>
 __device__ __forceinline__ T mul_add(T a, T b, T c, T d) {
   return fma(a, b, c * d);
@@ -179,6 +175,10 @@ template <typename T>
 __device__ __forceinline__ T mul_sub(T a, T b, T c, T d) {
   return fma(a, b, -(c * d));
 }
+// a product that is never fused into a later addition
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // a state value set that is physical: rho > 0, p > 0 and E finite.  With
 // rho > 0, p = (gamma - 1) (E - |m|^2 / (2 rho)) > 0 is 2 E rho > |m|^2,
 // which needs no division.  In FP64 only that test runs on the FP64 pipe: the
